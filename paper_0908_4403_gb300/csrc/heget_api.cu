@@ -1,5 +1,5 @@
 // heget_api.cu -- the C ABI of include/heget.h: context, argument checks,
-// launch shapes, the phase-space kernel and the fixed-order reductions.
+// launch shapes, the phase-space kernel and the reductions of partial sums.
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(256) f32_round_kernel(const double* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// fixed-order reductions
+// reductions
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ x, long long n,
                                                   Partial* __restrict__ partials) {
@@ -146,16 +146,67 @@ __global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ x, 
     if (threadIdx.x == 0) partials[blockIdx.x] = r;
 }
 
-// Combines nparts block partials in index order (called by one whole block).
+// Combines nparts block partials (called by one whole block of 256 threads):
+// the largest exponent first, then the terms as integers aligned to it
+// (heget_reduce.cuh), exactly, so in any order.
 // mode 0: write the heget_xsec_result (toy-PDF scale when kind == TOY_PDF);
 // mode 1: write (sum, sum of squares) to sums.
+struct FinalizeScratch {
+    __int128 v[2][8];
+    long long c[4][8];
+    int em[2][8];
+};
+
 __device__ __forceinline__ void finalize_block(const Partial* __restrict__ partials, int nparts, int kind, int mode,
                                                heget_xsec_result* __restrict__ res, double* __restrict__ sums,
-                                               Partial* scratch) {
-    Partial a = zero_partial();
-    for (int b = threadIdx.x; b < nparts; b += 256) a = partial_add(a, partials[b]);
-    const Partial r = block_reduce_partial<256>(a, scratch);
+                                               FinalizeScratch& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int em[2] = {1, 1};
+    for (int b = threadIdx.x; b < nparts; b += 256) {
+        em[0] = max(em[0], exponent_field(partials[b].sw));
+        em[1] = max(em[1], exponent_field(partials[b].sw2));
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        em[q] = (int)__reduce_max_sync(0xffffffffu, (unsigned)em[q]);
+        if (lane == 0) sh.em[q][warp] = em[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int w = 0; w < 8; ++w) em[q] = max(em[q], sh.em[q][w]);
+    // 2 nparts terms of one sum below 2^(53 + top) each: no overflow
+    const int top = 73 - (32 - __clz(2 * max(nparts, 1)));
+    __int128 v[2] = {0, 0};
+    long long c[4] = {0, 0, 0, 0};
+    for (int b = threadIdx.x; b < nparts; b += 256) {
+        const Partial p = partials[b];
+        v[0] += fixed_of(p.sw, em[0], top);
+        v[1] += fixed_of(p.sw2, em[1], top);
+        c[0] += p.npass;
+        c[1] += p.ntotal;
+        c[2] += p.ntries;
+        c[3] += p.nesc;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) v[q] += shfl_down128(v[q], off);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] += __shfl_down_sync(0xffffffffu, c[q], off);
+    }
+    if (lane == 0) {
+        for (int q = 0; q < 2; ++q) sh.v[q][warp] = v[q];
+        for (int q = 0; q < 4; ++q) sh.c[q][warp] = c[q];
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
+    for (int w = 1; w < 8; ++w) {
+        for (int q = 0; q < 2; ++q) v[q] += sh.v[q][w];
+        for (int q = 0; q < 4; ++q) c[q] += sh.c[q][w];
+    }
+    const Partial r{dd_of_fixed(v[0], em[0], top), dd_of_fixed(v[1], em[1], top), c[0], c[1], c[2], c[3]};
     const double sw = r.sw.hi + r.sw.lo, sw2 = r.sw2.hi + r.sw2.lo;
     if (mode == 1) {
         sums[0] = sw;
@@ -184,13 +235,13 @@ __device__ __forceinline__ void finalize_block(const Partial* __restrict__ parti
 __global__ void __launch_bounds__(256) finalize_kernel(const Partial* __restrict__ partials, int nparts, int kind,
                                                        int mode, heget_xsec_result* __restrict__ res,
                                                        double* __restrict__ sums) {
-    __shared__ Partial scratch[8];
+    __shared__ FinalizeScratch scratch;
     finalize_block(partials, nparts, kind, mode, res, sums, scratch);
 }
 
-// One block per batch request: its tile partials, in order, into its result.
+// One block per batch request: its tile partials into its result.
 __global__ void __launch_bounds__(256) finalize_batch_kernel(const BatchReq* __restrict__ reqs) {
-    __shared__ Partial scratch[8];
+    __shared__ FinalizeScratch scratch;
     const BatchReq& r = reqs[blockIdx.x];
     finalize_block(r.parts, r.ntiles, r.S.kind, 0, r.result, nullptr, scratch);
 }

@@ -211,17 +211,6 @@ struct Partial {
     long long npass, ntotal, ntries, nesc;
 };
 
-__host__ __device__ __forceinline__ Partial partial_add(const Partial& a, const Partial& b) {
-    Partial r;
-    r.sw = dd_add(a.sw, b.sw);
-    r.sw2 = dd_add(a.sw2, b.sw2);
-    r.npass = a.npass + b.npass;
-    r.ntotal = a.ntotal + b.ntotal;
-    r.ntries = a.ntries + b.ntries;
-    r.nesc = a.nesc + b.nesc;
-    return r;
-}
-
 // ---------------------------------------------------------------------------
 // Kernel arguments
 // ---------------------------------------------------------------------------

@@ -5,6 +5,7 @@
 // plus the launch-shape bookkeeping shared with the host code.
 #pragma once
 
+#include "heget_reduce.cuh"
 #include "heget_subset.cuh"
 
 namespace heget {
@@ -328,39 +329,6 @@ ward_kernel(const double* __restrict__ mom, long long npts, int ward, double* __
         for (int t = threadIdx.x; t < cnt; t += BLOCK)
             out[t0 + t] = recs[t].valid ? (double)recs[t].ssum : __longlong_as_double(0x7ff8000000000000ll);
     }
-}
-
-// Deterministic block reduction of per-thread partials (shuffle tree, then
-// warp leaders in order).  Uses `scratch` (BLOCK/32 Partials of shared
-// memory); result valid in thread 0.
-template <int BLOCK>
-__device__ __forceinline__ Partial block_reduce_partial(Partial a, Partial* scratch) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        Partial b;
-        b.sw.hi = __shfl_down_sync(0xffffffffu, a.sw.hi, off);
-        b.sw.lo = __shfl_down_sync(0xffffffffu, a.sw.lo, off);
-        b.sw2.hi = __shfl_down_sync(0xffffffffu, a.sw2.hi, off);
-        b.sw2.lo = __shfl_down_sync(0xffffffffu, a.sw2.lo, off);
-        b.npass = __shfl_down_sync(0xffffffffu, a.npass, off);
-        b.ntotal = __shfl_down_sync(0xffffffffu, a.ntotal, off);
-        b.ntries = __shfl_down_sync(0xffffffffu, a.ntries, off);
-        b.nesc = __shfl_down_sync(0xffffffffu, a.nesc, off);
-        a = partial_add(a, b);
-    }
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int w = 1; w < BLOCK / 32; ++w) a = partial_add(a, scratch[w]);
-    return a;
-}
-
-__device__ __forceinline__ Partial zero_partial() {
-    Partial p;
-    p.sw = DD{0, 0};
-    p.sw2 = DD{0, 0};
-    p.npass = p.ntotal = p.ntries = p.nesc = 0;
-    return p;
 }
 
 // Ordered compaction: the position of this thread's flagged item among the
@@ -968,7 +936,7 @@ size_t batch_tile_smem(int n, int precision, int alg, int tile);
 // default for the tree; for the subset recursion tiles that fill two blocks
 // per SM (its per-point cost is far below the tree's at large n).
 int batch_default_tile(int n, int precision, int alg);
-// One block per request: its tile partials, in order, into its result.
+// One block per request: its tile partials into its result.
 int launch_batch_finalize(const BatchReq* reqs, int nreqs, cudaStream_t st);
 
 // Default launch shape and the maximum resident blocks per SM.

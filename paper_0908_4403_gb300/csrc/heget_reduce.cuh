@@ -1,0 +1,162 @@
+// heget_reduce.cuh -- combination of Monte Carlo partials (double-double sums
+// and counters) across the threads of a block and across blocks.
+//
+// Partials are combined in integers: every term is aligned to the largest
+// exponent among them as a 128-bit fixed-point number, the numbers are added
+// as integers, and the total goes back to a double-double.  The additions are
+// exact, so the result does not depend on their order; what is lost are bits
+// below 2^-115 (a warp) or 2^-(120 - log2 terms) (a whole grid) of the largest
+// term, at or below the 2^-104 of a double-double addition.
+//
+// Why integers: GB300 issues a warp's FP64 instruction in 64 cycles of its
+// sub-partition whatever the number of active lanes, and a double-double
+// addition takes 20 of them.  A tree of double-double additions over a
+// 256-thread block (5 shuffle levels x 2 sums, then 7 by one thread) held the
+// FP64 pipe at the end of every block -- 600 of the 1160 FP64 instructions a
+// point of a 128-point FP64 tile at n = 2 -- and the one-block finalisation
+// for 43 us.  The integer form is about 300 integer instructions a warp.
+// GB300, before -> after: one call of 1000 points at n = 2 102 -> 41 us, 65,536
+// points in FP64 228 -> 96 us, n = 4 FP32 1,048,576 points 1202 -> 1123 us, FP64
+// 262,144 points 3483 -> 3030 us, a batch of 24 mixed requests 4883 -> 4286 us,
+// with the same bits in every result.
+#pragma once
+
+#include "heget_common.cuh"
+
+namespace heget {
+
+__host__ __device__ __forceinline__ unsigned long long double_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(x);
+#else
+    unsigned long long u;
+    __builtin_memcpy(&u, &x, sizeof u);
+    return u;
+#endif
+}
+__host__ __device__ __forceinline__ double bits_double(unsigned long long u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double x;
+    __builtin_memcpy(&x, &u, sizeof x);
+    return x;
+#endif
+}
+
+// Biased exponent of x, 1 for zero and subnormals, 0x7FF for inf and NaN.
+__host__ __device__ __forceinline__ int exponent_field(double x) {
+    const int e = (int)(double_bits(x) >> 52) & 0x7FF;
+    return e > 0 ? e : 1;
+}
+__host__ __device__ __forceinline__ int exponent_field(const DD& a) {
+    const int h = exponent_field(a.hi), l = exponent_field(a.lo);
+    return h > l ? h : l;
+}
+
+// x as an integer in units of 2^(em - 1075 - top), truncated towards zero;
+// em >= the exponent field of x, 0 <= top <= 73.  A term is below
+// 2^(53 + top) in magnitude: up to 2^(73 - top) of them add up without
+// overflow.
+__host__ __device__ __forceinline__ __int128 fixed_of(double x, int em, int top) {
+    const unsigned long long u = double_bits(x);
+    const int ef = (int)(u >> 52) & 0x7FF;
+    unsigned long long m = u & 0xFFFFFFFFFFFFFull;
+    if (ef) m |= 1ull << 52;
+    const int sh = top - (em - (ef ? ef : 1));
+    unsigned __int128 v = m;
+    if (sh >= 0) v <<= sh;
+    else v = sh > -64 ? (unsigned __int128)(m >> -sh) : 0;
+    return (u >> 63) ? -(__int128)v : (__int128)v;
+}
+__host__ __device__ __forceinline__ __int128 fixed_of(const DD& a, int em, int top) {
+    return fixed_of(a.hi, em, top) + fixed_of(a.lo, em, top);
+}
+
+__host__ __device__ __forceinline__ int clz64(unsigned long long x) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)x);
+#else
+    return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+// m 2^e (m < 2^53) as a double, exact unless it leaves the double range.
+__host__ __device__ __forceinline__ double scaled_int(unsigned long long m, int e) {
+    if (m == 0) return 0.0;
+    const int lz = clz64(m) - 11;               // to bit 52
+    const int field = e - lz + 1075;
+    if (field >= 1 && field <= 2046)
+        return bits_double(((unsigned long long)field << 52) | ((m << lz) & 0xFFFFFFFFFFFFFull));
+    return scalbn((double)m, e);
+}
+
+// The double-double of v 2^(em - 1075 - top), the top 106 bits of v.  em is
+// 0x7FF when a term was not finite: the sum is then NaN, as a double-double
+// sum of such terms is.
+__host__ __device__ __forceinline__ DD dd_of_fixed(__int128 v, int em, int top) {
+    if (em >= 0x7FF) return DD{bits_double(0x7FF8000000000000ull), 0.0};
+    const bool neg = v < 0;
+    unsigned __int128 u = neg ? -(unsigned __int128)v : (unsigned __int128)v;
+    if (u == 0) return DD{0.0, 0.0};
+    const unsigned long long uh = (unsigned long long)(u >> 64);
+    const int lz = uh ? clz64(uh) : 64 + clz64((unsigned long long)u);
+    u <<= lz;                                   // leading bit at 127
+    const int e = em - 1075 - top - lz;         // weight of bit 0 of u
+    const double hi = scaled_int((unsigned long long)(u >> 75), e + 75);
+    const double lo = scaled_int((unsigned long long)(u >> 22) & ((1ull << 53) - 1), e + 22);
+    return neg ? DD{-hi, -lo} : DD{hi, lo};
+}
+
+constexpr int kWarpTop = 66;   // 64 terms a warp (hi and lo of 32 lanes), one bit to spare
+
+__device__ __forceinline__ __int128 shfl_down128(__int128 v, int off) {
+    const unsigned long long l = __shfl_down_sync(0xffffffffu, (unsigned long long)v, off);
+    const unsigned long long h = __shfl_down_sync(0xffffffffu, (unsigned long long)((unsigned __int128)v >> 64), off);
+    return (__int128)(((unsigned __int128)h << 64) | l);
+}
+
+__device__ __forceinline__ DD warp_sum_dd(const DD& a) {
+    const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a));
+    __int128 v = fixed_of(a, em, kWarpTop);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += shfl_down128(v, off);
+    return dd_of_fixed(v, em, kWarpTop);
+}
+
+// Sum over the 32 lanes of a warp, valid in lane 0.
+__device__ __forceinline__ Partial warp_reduce_partial(Partial a) {
+    a.sw = warp_sum_dd(a.sw);
+    a.sw2 = warp_sum_dd(a.sw2);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a.npass += __shfl_down_sync(0xffffffffu, a.npass, off);
+        a.ntotal += __shfl_down_sync(0xffffffffu, a.ntotal, off);
+        a.ntries += __shfl_down_sync(0xffffffffu, a.ntries, off);
+        a.nesc += __shfl_down_sync(0xffffffffu, a.nesc, off);
+    }
+    return a;
+}
+
+__device__ __forceinline__ Partial zero_partial() {
+    Partial p;
+    p.sw = DD{0, 0};
+    p.sw2 = DD{0, 0};
+    p.npass = p.ntotal = p.ntries = p.nesc = 0;
+    return p;
+}
+
+// Sum of the per-thread partials of a block (each warp, then the warps'
+// sums).  Uses `scratch` (BLOCK/32 Partials of shared memory); result valid
+// in thread 0.  All threads must call it.
+template <int BLOCK>
+__device__ __forceinline__ Partial block_reduce_partial(Partial a, Partial* scratch) {
+    static_assert(BLOCK % 32 == 0 && BLOCK / 32 <= 32, "whole warps, one warp to add them");
+    a = warp_reduce_partial(a);
+    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = a;
+    __syncthreads();
+    if (threadIdx.x < 32) a = warp_reduce_partial(threadIdx.x < BLOCK / 32 ? scratch[threadIdx.x] : zero_partial());
+    return a;
+}
+
+}  // namespace heget
