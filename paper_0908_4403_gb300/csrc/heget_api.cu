@@ -369,7 +369,8 @@ Physics physics_of(const heget_params& p, int n) {
     ph.sinh_eta = std::sinh(p.eta_max);
     ph.cosh_eta = std::cosh(p.eta_max);
     ph.sinh_dr = p.dr_min > 0 ? std::sinh(p.dr_min) : 0.0;
-    ph.cos_dr = p.dr_min > 0 ? std::cos(p.dr_min) : 1.0;
+    // (cos d phi < cos R needs R < pi: beyond it no pair is far in phi alone)
+    ph.cos_dr = p.dr_min > 0 ? (p.dr_min < M_PI ? std::cos(p.dr_min) : -2.0) : 1.0;
     return ph;
 }
 

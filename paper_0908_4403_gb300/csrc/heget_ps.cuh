@@ -483,7 +483,9 @@ __device__ __forceinline__ int pass_cuts(const MomView& p, double ey, double iey
                 const double s2 = sh * sh / pp2, t2 = cr * cr / (dot * dot);
                 const double a = 1.0 - s2 * (1.0 / 6.0), b = 1.0 - t2 * (1.0 / 3.0);
                 const double hi = s2 + t2, lo = s2 * a * a + t2 * b * b;
-                if (lo > R2 * (1.0 + 1e-12)) {
+                if (!(a > 0 && b > 0)) {
+                    exact = true;   // wide cuts (R beyond about 1): the lower bounds do not hold
+                } else if (lo > R2 * (1.0 + 1e-12)) {
                     // Delta R > R: the pair passes
                 } else if (hi < R2 * (1.0 - 1e-12)) {
                     ok = false;
