@@ -505,86 +505,104 @@ __device__ __forceinline__ int pass_cuts(const MomView& p, double ey, double iey
     return ok ? 1 : 0;
 }
 
-// FP32 prefilter of the cut decisions.  Each test of pass_cuts is decided in
-// FP32 when the FP32 value lies clearly on one side of the boundary, and the
-// point falls back to the FP64 pass_cuts otherwise, so every decision equals
-// the FP64 one.  Error bounds (u = 2^-24): the components convert with
-// relative error u; a product or sum of two such terms carries at most a
-// few u relative to the magnitudes involved.  Margins are 64 u relative for
-// the single-photon tests (no cancellation) and 32 u times the sum of the
-// term magnitudes for the pair quantities sinh(d eta) pT pT and
-// cos(d phi) pT pT, which cancel.  Only the rare close pairs (which need
-// the exact Delta R) and near-boundary tests reach FP64.
-struct Tri {   // a decision: certain (true / false) or undecided
-    bool ok, sure;
-};
-
-// v < a w with w = sqrt(w2) >= 0, from FP32 values v2 = v^2, r2 = a^2 w2
-// carrying relative error <= rel, and exact signs of v and a.
-__device__ __forceinline__ Tri lt_scaled_f(bool vneg, bool apos, float v2, float r2, float rel) {
-    const bool lt = v2 < r2 * (1.0f - rel), gt = v2 > r2 * (1.0f + rel);
-    if (apos) return vneg ? Tri{true, true} : Tri{lt, lt || gt};
-    return vneg ? Tri{gt, lt || gt} : Tri{false, true};
+// x as a float for the FP32 cut decisions: truncated towards zero (relative
+// error below 2^-23; zero below the normal float range) by three integer
+// operations on the bits.  x must be below the float range's end.
+__device__ __forceinline__ float f32_cut(double x) {
+    const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+    const unsigned int f = __funnelshift_l(lo, hi, 3) - (384u << 23);   // 9 exponent bits rebased by 896 mod 512
+    const bool tiny = (hi & 0x7FFFFFFFu) < 0x38100000u;
+    return tiny ? 0.0f : __uint_as_float((f & 0x7FFFFFFFu) | (hi & 0x80000000u));
 }
 
+// The cut decisions in FP32 wherever FP32 settles them: the same decisions as
+// pass_cuts, which decides the points that stay open.  With u = 2^-24, the
+// truncated components carry 2 u.  Rapidities enter through the light-cone
+// components p+ = E + pz, p- = pT^2 / p+ (for pz >= 0; the other way round
+// below 0), which do not cancel:
+//   eta + y < E  <=>  p+ e^y < e^2E p- e^-y,
+//   sinh(eta_i - eta_j) pT_i pT_j = (p+_i p-_j - p-_i p+_j) / 2,
+// all terms within about 20 u, so 64 u of relative margin (32 u of the terms'
+// magnitudes for the two sides of the difference, 16 u for cos(d phi) pT pT)
+// is safe.  A pair that is not surely far in eta or phi takes asinhf and
+// atan2f (3 ulp each): d eta and d phi within 32 u absolute, and Delta R^2
+// open only within 2 (d eta + d phi) 32 u of R^2.  About 3e-4 of the points
+// stay open (n = 4, toy PDF).
+//
+// Bound: the FP64 tests cost 24 + 10 n (n - 1) / 2 FP64 instructions a point
+// (90 of 545 at n = 4) at 64 cycles each per warp; these cost about 70 n + 20
+// n (n - 1) / 2 FP32 and integer instructions at 1 - 2 cycles.  GB300, before ->
+// after: n = 4 step of 1,048,576 points 1123 -> 1012 us, phase space of 500,000
+// points at n = 5 668 -> 454 us.
+//
+// FP32 holds the squares and fourth powers of momenta of 1e-2 .. 1e8 GeV
+// events and the cuts' e^2E and sinh^2 R: other events and cuts are left to
+// pass_cuts, and so is a photon whose pT^2 FP32 cannot hold accurately.
 template <int N>
-__device__ __forceinline__ int pass_cuts_fast(const MomView& p, double ey, double iey, const Physics& ph) {
+__device__ __forceinline__ int pass_cuts_fast(const MomView& p, double rs, double ey, double iey, const Physics& ph) {
     constexpr float kU = 5.9604645e-8f;   // 2^-24
-    const double shy = 0.5 * (ey - iey), chy = 0.5 * (ey + iey);
-    const double s_hi = ph.sinh_eta * chy - ph.cosh_eta * shy;    // sinh(E - y)
-    const double s_lo = -ph.sinh_eta * chy - ph.cosh_eta * shy;   // sinh(-E - y)
-    const float shi_f = f32_rn(s_hi), slo_f = f32_rn(s_lo);
-    const float shi2 = shi_f * shi_f, slo2 = slo_f * slo_f;
-    const float ptmin2 = f32_rn(ph.pt_min * ph.pt_min);
-    float x[N], y[N], z[N], e[N], pt2[N];
-    bool ok = true, sure = true;
+    if (!(rs > 1e-2 && rs < 1e8 && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12))
+        return pass_cuts<N>(p, ey, iey, ph);
+    constexpr float kLo = 1.0f - 64.0f * kU, kHi = 1.0f + 64.0f * kU;
+    const float eyf = f32_cut(ey), ieyf = f32_cut(iey);
+    const float eE = f32_cut(ph.sinh_eta) + f32_cut(ph.cosh_eta), e2E = eE * eE;
+    const float ptmin2 = f32_cut(ph.pt_min) * f32_cut(ph.pt_min);
+    float x[N], y[N], pp[N], pm[N], pt2[N];
+    bool fail = false, open = false;   // some test surely fails; some test is not decided
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        e[i] = f32_rn(p(i, 0));
-        x[i] = f32_rn(p(i, 1));
-        y[i] = f32_rn(p(i, 2));
-        z[i] = f32_rn(p(i, 3));
+        const float e = f32_cut(p(i, 0)), z = f32_cut(p(i, 3));
+        x[i] = f32_cut(p(i, 1));
+        y[i] = f32_cut(p(i, 2));
         pt2[i] = x[i] * x[i] + y[i] * y[i];
-        const bool gt = pt2[i] > ptmin2 * (1.0f + 64.0f * kU), le = pt2[i] < ptmin2 * (1.0f - 64.0f * kU);
-        sure = sure && (gt || le);
-        ok = ok && gt;
-        const float z2 = z[i] * z[i];
-        const Tri hi = lt_scaled_f(z[i] < 0.0f, shi_f >= 0.0f, z2, shi2 * pt2[i], 64.0f * kU);
-        const Tri lo = lt_scaled_f(z[i] > 0.0f, -slo_f >= 0.0f, z2, slo2 * pt2[i], 64.0f * kU);
-        sure = sure && hi.sure && lo.sure;
-        ok = ok && hi.ok && lo.ok;
+        const float big = e + fabsf(z), small = __fdividef(pt2[i], big);
+        pp[i] = z < 0.0f ? small : big;
+        pm[i] = z < 0.0f ? big : small;
+        const bool held = pt2[i] > 1e-30f;
+        fail = fail || pt2[i] < ptmin2 * kLo;
+        open = open || !(held && pt2[i] > ptmin2 * kHi);
+        const float a = pp[i] * eyf, b = pm[i] * ieyf;
+        fail = fail || (held && (a * kLo > e2E * b || b * kLo > e2E * a));
+        open = open || !(a * kHi < e2E * b && b * kHi < e2E * a);
     }
-    bool close = false;
+    unsigned close = 0;
     if (ph.dr_min > 0) {
-        const float sdr2 = f32_rn(ph.sinh_dr * ph.sinh_dr), cdr = f32_rn(ph.cos_dr);
+        const float sdr = f32_cut(ph.sinh_dr), sdr2 = sdr * sdr, cdr = f32_cut(ph.cos_dr);
 #pragma unroll
         for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int j = i + 1; j < N; ++j) {
                 const float pp2 = pt2[i] * pt2[j];
-                const float sh = z[i] * e[j] - z[j] * e[i];
-                const float esh = 32.0f * kU * (fabsf(z[i] * e[j]) + fabsf(z[j] * e[i]));
-                const float dot = x[i] * x[j] + y[i] * y[j];
-                const float edot = 32.0f * kU * (fabsf(x[i] * x[j]) + fabsf(y[i] * y[j]));
-                const float ash = fabsf(sh);
-                // far in eta: sh^2 > sdr2 pp2, certain if (|sh| - esh)^2 beats it
-                const float T = sdr2 * pp2;
-                const bool eta_far = ash > esh && (ash - esh) * (ash - esh) > T * (1.0f + 64.0f * kU);
-                const bool eta_near = (ash + esh) * (ash + esh) < T * (1.0f - 64.0f * kU);
-                // far in phi: dot < cos_dr pT pT
-                const float c = cdr * sqrtf(pp2);
-                const float ec = 64.0f * kU * fabsf(c);
-                const bool phi_far = dot + edot < c - ec;
-                const bool phi_near = dot - edot > c + ec;
-                const bool far = eta_far || phi_far;
-                sure = sure && (far || (eta_near && phi_near));
-                close = close || (!far && eta_near && phi_near);
+                const float u = pp[i] * pm[j], v = pm[i] * pp[j];
+                const float sh = fabsf(u - v) - 32.0f * kU * (u + v);   // twice |sinh(d eta)| pT pT, from below
+                const float xx = x[i] * x[j], yy = y[i] * y[j];
+                const float dot = xx + yy + 16.0f * kU * (fabsf(xx) + fabsf(yy));   // from above
+                const float c = cdr * (pp2 * rsqrtf(pp2));
+                const bool far = (sh > 0.0f && sh * sh * 0.25f > sdr2 * pp2 * kHi) || dot < c - 64.0f * kU * fabsf(c);
+                close |= (far ? 0u : 1u) << pair_index<N>(i, j);
             }
     }
-    // undecided tests, and the close pairs (which need the exact Delta R),
-    // go to the FP64 decision
-    if (!sure || (ok && close)) return pass_cuts<N>(p, ey, iey, ph);
-    return ok ? 1 : 0;
+    if (fail) return 0;
+    const float R = f32_cut(ph.dr_min), R2 = R * R;
+    while (close) {
+        int q = __ffs(close) - 1, i = 0;
+        close &= close - 1;
+        while (q >= N - 1 - i) q -= N - 1 - i++;
+        const int j = i + 1 + q;
+        const float xi = f32_cut(p(i, 1)), yi = f32_cut(p(i, 2)), zi = f32_cut(p(i, 3));
+        const float xj = f32_cut(p(j, 1)), yj = f32_cut(p(j, 2)), zj = f32_cut(p(j, 3));
+        const float ti = xi * xi + yi * yi, tj = xj * xj + yj * yj;
+        const float bi = f32_cut(p(i, 0)) + fabsf(zi), bj = f32_cut(p(j, 0)) + fabsf(zj);
+        const float si = __fdividef(ti, bi), sj = __fdividef(tj, bj);
+        const float u = (zi < 0.0f ? si : bi) * (zj < 0.0f ? bj : sj), v = (zi < 0.0f ? bi : si) * (zj < 0.0f ? sj : bj);
+        const float deta = asinhf(0.5f * fabsf(u - v) * rsqrtf(ti * tj));
+        const float dphi = atan2f(fabsf(xi * yj - yi * xj), xi * xj + yi * yj);
+        const float d2 = deta * deta + dphi * dphi;
+        const float m = 64.0f * kU * (deta + dphi + 64.0f * kU) + 8.0f * kU * R2;
+        if (d2 < R2 - m) return 0;
+        open = open || !(d2 > R2 + m);
+    }
+    return open ? pass_cuts<N>(p, ey, iey, ph) : 1;
 }
 
 // Event i of stream `seed` from its sampler draws d: sqrt(s-hat), RAMBO
@@ -594,11 +612,7 @@ __device__ __forceinline__ void generate_from(const PointRng& rng, const SampleD
                                               const Physics& ph, const MomView& v, EventInfo& ev) {
     sample_finish(S, d, ev);
     rambo<N>(rng, ev.rs, v);
-    // the FP32 prefilter keeps 5n floats per photon set live in the producer
-    // threads: a gain up to n = 3 (+22 % at n = 2 on GB300), a loss above
-    // (at n = 4 1 % slower even with 124 registers a producer thread)
-    if constexpr (N <= 3) ev.mask = ev.ok ? pass_cuts_fast<N>(v, ev.ey, ev.iey, ph) : 0;
-    else ev.mask = ev.ok ? pass_cuts<N>(v, ev.ey, ev.iey, ph) : 0;
+    ev.mask = ev.ok ? pass_cuts_fast<N>(v, ev.rs, ev.ey, ev.iey, ph) : 0;
 }
 
 template <int N>
