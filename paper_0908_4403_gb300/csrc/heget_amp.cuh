@@ -651,6 +651,13 @@ __device__ __forceinline__ float sel_weight(int hsel, unsigned lam, float w) {
 }
 
 
+// |A|^2 with the additions' order and the fused operation written out, so that
+// it has the same bits in every kernel that it is inlined into.
+template <class R>
+__device__ __forceinline__ R norm2(R re, R im) {
+    return fmad<R>(re, re, im * im);
+}
+
 // Lane coordinates in a round: group or slot, point slot, lane bits.
 template <int N, int BLOCK, int HB, int G>
 struct LaneId {
@@ -739,7 +746,7 @@ __device__ __forceinline__ void amplitude_rounds_lanes(unsigned char* table_smem
         combine_groups<R, N, BLOCK, BAR, G>(tb, id, are, aim);
         // a sampled helicity (PointRec::hsel): only the selected lane counts
         const int hsel = active ? recs[base + id.slot].hsel : -1;
-        const R v = (are[0] * are[0] + aim[0] * aim[0]) * R(sel_weight<N>(hsel, (unsigned)id.hl, wh));
+        const R v = norm2(are[0], aim[0]) * R(sel_weight<N>(hsel, (unsigned)id.hl, wh));
         const R s = point_reduce<R, N, BLOCK, BAR, G, false>(tb, v);
         if (id.g == 0 && id.hl == 0 && id.slot < rc) recs[base + id.slot].ssum = s;
         group_sync<BAR, BLOCK>();

@@ -75,7 +75,7 @@ phase_space_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, P
                    double* __restrict__ w, double* __restrict__ rs_out, double* __restrict__ y_out,
                    uint8_t* __restrict__ mask_out, int32_t* __restrict__ tries_out) {
     __shared__ double stage[N * kMomSlots * kPsBlock];
-    __shared__ double rs_s[kPsBlock];
+    __shared__ double rs_s[kPsBlock], sc_s[kPsBlock];   // sqrt(s-hat), and the momenta's scale to GeV
     constexpr int ROW = (N + 2) * 4;
     for (long long j0 = (long long)blockIdx.x * kPsBlock; j0 < npts; j0 += (long long)gridDim.x * kPsBlock) {
         const int cnt = (int)min((long long)kPsBlock, npts - j0);
@@ -88,7 +88,8 @@ phase_space_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, P
             rs_s[t] = ev.rs;
             if (w) w[j] = ev.ok ? phase_space_weight<N>(ev.rs * ev.rs) : 0.0;
             if (rs_out) rs_out[j] = ev.rs;
-            if (y_out) y_out[j] = (S.kind == HEGET_SAMPLER_TOY_PDF && ev.ok) ? 0.5 * log(ev.x1 / ev.x2) : 0.0;
+            sc_s[t] = ev.rs * ev.iM;
+            if (y_out) y_out[j] = (S.kind == HEGET_SAMPLER_TOY_PDF && ev.ok) ? event_rapidity(ev) : 0.0;
             if (mask_out) mask_out[j] = (uint8_t)ev.mask;
             if (tries_out) tries_out[j] = ev.tries;
         }
@@ -99,7 +100,7 @@ phase_space_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, P
                 const int p = e / ROW, c = e - p * ROW, a = c >> 2, m = c & 3;
                 double val;
                 if (a >= 2) {
-                    val = stage[(kMomSlots * (a - 2) + m) * kPsBlock + p];
+                    val = stage[(kMomSlots * (a - 2) + m) * kPsBlock + p] * sc_s[p];
                 } else {   // p1 = (rs/2)(1,0,0,1), p2 = (rs/2)(1,0,0,-1)
                     const double h = 0.5 * rs_s[p];
                     val = m == 0 ? h : (m == 3 ? (a == 0 ? h : -h) : 0.0);

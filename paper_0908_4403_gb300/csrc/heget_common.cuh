@@ -162,13 +162,6 @@ struct PointRng {
     __device__ __forceinline__ U4 words(uint32_t tag, uint32_t b) const {
         return philox4x32_10(U4{ilo, ihi, b, tag}, k0, k1);
     }
-    // both draws of block b of stream `tag`
-    __device__ __forceinline__ void pair(uint32_t tag, uint32_t b, double& u0,
-                                         double& u1) const {
-        const U4 w = words(tag, b);
-        u0 = u01_from_words(w.x, w.y);
-        u1 = u01_from_words(w.z, w.w);
-    }
 };
 
 // ---------------------------------------------------------------------------
@@ -187,9 +180,8 @@ __host__ __device__ __forceinline__ DD dd_add_d(DD a, double b) {
     double s, e;
     two_sum(a.hi, b, s, e);
     e += a.lo;
-    double h, l;
-    two_sum(s, e, h, l);
-    return DD{h, l};
+    const double h = s + e;   // |s| >= |e| (or s = 0): Dekker's fast two-sum is exact
+    return DD{h, e - (h - s)};
 }
 
 __host__ __device__ __forceinline__ DD dd_add(DD a, DD b) {

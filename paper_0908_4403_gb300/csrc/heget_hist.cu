@@ -68,12 +68,13 @@ hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics 
         if (tid < cnt) {
             EventInfo ev;
             generate_event<N>(seed, (uint64_t)(i0 + t0 + tid), S, ph, v, ev);
-            const double y = (S.kind == HEGET_SAMPLER_TOY_PDF && ev.ok) ? 0.5 * log(ev.x1 / ev.x2) : 0.0;
+            const double y = (S.kind == HEGET_SAMPLER_TOY_PDF && ev.ok) ? event_rapidity(ev) : 0.0;
+            const double scale = ev.rs * ev.iM;
             // the photon observables replace the momenta in the point's column:
             // slot 0 pT, 1 eta (lab), 2 phi
 #pragma unroll 1
             for (int i = 0; i < N; ++i) {
-                const double px = v(i, 1), py = v(i, 2), pz = v(i, 3);
+                const double px = v(i, 1) * scale, py = v(i, 2) * scale, pz = v(i, 3) * scale;
                 const double pt = sqrt(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)));
                 v(i, 0) = pt;
                 v(i, 1) = asinh(pz / pt) + y;

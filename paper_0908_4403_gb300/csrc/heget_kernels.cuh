@@ -390,7 +390,8 @@ __device__ __forceinline__ void xsec_tile(unsigned char* smem, int tile, uint64_
         if (pass) {
             recs[npass + pos].idx = t;
             recs[npass + pos].hsel = point_hsel<N>(ph, seed, (uint64_t)(first + t));
-            recs[npass + pos].fac = ev.irs;   // 1/sqrt(s-hat) until the record is built
+            recs[npass + pos].fac = ev.iM;   // 1/M and sqrt(s-hat) until the record is built
+            recs[npass + pos].wfac = ev.rs;
         }
         npass += tot;
     }
@@ -398,7 +399,7 @@ __device__ __forceinline__ void xsec_tile(unsigned char* smem, int tile, uint64_
     // records built one per thread in compacted order: every lane busy
     for (int c = threadIdx.x; c < npass; c += BLOCK) {
         PointRec<R, N>& rec = recs[c];
-        pass_to_rec<R, N>(MomView{stage + rec.idx, tile, kMomSlots}, rec.fac, ph, rec);
+        pass_to_rec<R, N>(MomView{stage + rec.idx, tile, kMomSlots}, rec.fac, rec.wfac, ph, rec);
     }
     if constexpr (N >= 6) {
         __syncthreads();   // the staged momenta are scaled in place by pass_to_rec
@@ -515,7 +516,7 @@ xsec_escalate_kernel(uint64_t seed, long long i0, SamplerArgs S, Physics ph, int
             const MomView v{stage + t, tile, kMomSlots};
             EventInfo ev;
             generate_event<N>(seed, (uint64_t)esc.idx[base + c0 + t], S, ph, v, ev);
-            pass_to_rec<double, N>(v, ev.irs, ph, recs[t]);
+            pass_to_rec<double, N>(v, ev.iM, ev.rs, ph, recs[t]);
             recs[t].idx = t;
             recs[t].hsel = point_hsel<N>(ph, seed, (uint64_t)esc.idx[base + c0 + t]);
         }
@@ -821,13 +822,14 @@ xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physi
             if (pass) {
                 rs_ring[pos].idx = g;
                 rs_ring[pos].hsel = point_hsel<N>(ph, seed, (uint64_t)(i0 + t0 + g));
-                rs_ring[pos].fac = ev.irs;   // 1/sqrt(s-hat) until the record is built
+                rs_ring[pos].fac = ev.iM;   // 1/M and sqrt(s-hat) until the record is built
+                rs_ring[pos].wfac = ev.rs;
             }
             named_sync(kBarProducers, kWsStage);
             // records built one per producer in compacted order: every lane busy
             if (g < tot)
-                pass_to_rec<R, N>(MomView{stage + rs_ring[g].idx, kWsStage, kMomSlots}, rs_ring[g].fac, ph,
-                                  rs_ring[g]);
+                pass_to_rec<R, N>(MomView{stage + rs_ring[g].idx, kWsStage, kMomSlots}, rs_ring[g].fac, rs_ring[g].wfac,
+                                  ph, rs_ring[g]);
             if constexpr (N >= 6) {
                 named_sync(kBarProducers, kWsStage);   // scaled momenta in place
                 denominators_parallel<R, N, false, true>(rs_ring, tot, g, kWsStage, [&](int c, double& E1, double& E2, double& is) {

@@ -4,12 +4,15 @@
 // eqs. (9)-(10), and the per-point record the amplitude kernels consume.
 //
 // GB300 executes FP64 at about 1/64 of the FP32 rate, so this file keeps
-// FP64 for what needs it (RAMBO energies, angles and boosts; the Lorentz
-// invariants behind the propagator denominators; cut decisions) and avoids
-// FP64 transcendentals where an algebraic identity gives the same decision.
+// FP64 for what needs it (RAMBO's boost; the Lorentz invariants behind the
+// propagator denominators; cut decisions near a boundary): the isotropic
+// momenta come from integer arithmetic of more bits (heget_dir.cuh), the cuts
+// from FP32 where it decides, and square roots and reciprocals from FP32
+// estimates refined in FP64.
 #pragma once
 
 #include "heget_common.cuh"
+#include "heget_dir.cuh"
 #include "heget_logtab.h"
 #include "heget_sincostab.h"
 
@@ -131,13 +134,27 @@ __device__ __forceinline__ double toy_pdf_x_of(uint32_t wx, uint32_t wy) {
     return __dmul_rn(u, u);
 }
 
-// Scalars of one generated event; its photon momenta (GeV) live in a MomView.
-// ey, iey: e^y and e^-y of the partonic frame's rapidity y (1 for the fixed
-// and uniform samplers).
+// Scalars of one generated event.  Its photon momenta in a MomView are those
+// of RAMBO before the last scaling, with total (M, 0, 0, 0): times iM = 1/M
+// they are in units of sqrt(s-hat) = rs, times rs iM in GeV.  ua, ub: the
+// uniforms behind the toy PDF's fractions x = u^2, as integers u 2^53 (equal
+// for the other samplers), so that e^y = sqrt(x1 / x2) = ua / ub.
 struct EventInfo {
-    double rs, irs, ey, iey, x1, x2;
+    double rs, iM;
+    u64 ua, ub;
     int tries, ok, mask;
 };
+
+// The partonic frame's rapidity y = ln(x1 / x2) / 2 = ln ua - ln ub.
+__device__ __forceinline__ double event_rapidity(const EventInfo& ev) {
+    const __int128 d = (__int128)neg_log(ev.ub, 1ull << 53, kDirLog) - (__int128)neg_log(ev.ua, 1ull << 53, kDirLog);
+    const bool neg = d < 0;
+    const unsigned __int128 a = neg ? -(unsigned __int128)d : (unsigned __int128)d;   // y 2^72, below 2^80
+    const u64 h = (u64)(a >> 32), l = (u64)(u32)a << 32;
+    if ((h | l) == 0) return 0.0;
+    const int lz = clz128(h, l);
+    return double_of(lz ? shift_top(h, l, lz) : h, 32 - lz - 72, neg);
+}
 
 // Helicity sampling (the paper's events carry one random helicity
 // combination, Sec. 3): h = floor(2^(n+2) u) with u draw 0 of the helicity
@@ -213,37 +230,25 @@ __device__ __forceinline__ SampleDraw sample_draw(const SamplerArgs& S, const Po
     return d;
 }
 
-// sqrt(s-hat) and its inverse, the momentum fractions, the boost factors
-// e^+-y and the outer attempts from the draws.  With sqrt(s-hat) = 2 E
-// sqrt(x1 x2), e^y = sqrt(x1 / x2) = 2 E x1 / sqrt(s-hat) and e^-y = 2 E x2 /
-// sqrt(s-hat): one division serves all three.  y itself (a logarithm) is
-// left to callers that output it.
+// sqrt(s-hat) and the outer attempts from the draws: 2 E sqrt(x1 x2) = 2 E ua
+// ub, with the product of the uniforms rounded once.
 __device__ __forceinline__ void sample_finish(const SamplerArgs& S, const SampleDraw& d, EventInfo& ev) {
     ev.ok = d.ok();
     ev.tries = d.tries();
-    ev.ey = ev.iey = 1.0;
-    ev.x1 = ev.x2 = 1.0;
+    ev.ua = ev.ub = 1;
     if (S.kind == HEGET_SAMPLER_FIXED) {
         ev.rs = S.sqrt_s;
-        ev.irs = 1.0 / ev.rs;
-        return;
-    }
-    if (S.kind == HEGET_SAMPLER_UNIFORM) {
+    } else if (S.kind == HEGET_SAMPLER_UNIFORM) {
         ev.rs = S.lo + (S.hi - S.lo) * u01_from_words(d.ax, d.ay);
-        ev.irs = 1.0 / ev.rs;
-        return;
-    }
-    if (ev.ok) {
-        ev.x1 = toy_pdf_x_of(d.ax, d.ay);
-        ev.x2 = toy_pdf_x_of(d.bx, d.by);
-        ev.rs = 2.0 * S.e_beam * sqrt(ev.x1 * ev.x2);
+    } else if (ev.ok) {
+        ev.ua = u53_of_words(d.ax, d.ay);
+        ev.ub = u53_of_words(d.bx, d.by);
+        const unsigned __int128 P = (unsigned __int128)ev.ua * ev.ub;
+        const int lz = clz128((u64)(P >> 64), (u64)P);
+        ev.rs = 2.0 * S.e_beam * double_of(shift_top((u64)(P >> 64), (u64)P, lz), 64 - lz - 106, false);
     } else {
         ev.rs = S.floor;
     }
-    ev.irs = 1.0 / ev.rs;
-    const double h = 2.0 * S.e_beam * ev.irs;
-    ev.ey = ev.ok ? ev.x1 * h : 1.0;
-    ev.iey = ev.ok ? ev.x2 * h : 1.0;
 }
 
 // Photon momenta of one point held in shared memory: slot (a, m) at
@@ -341,53 +346,67 @@ __device__ __forceinline__ void sincos_2pi_words(uint32_t lo, uint32_t hi, doubl
     sp = a.y + fma(a.y, cm, a.x * s);
 }
 
-// RAMBO: n massless momenta with total (rs, 0, 0, 0).  Photon i uses draws
-// 4i..4i+3 of the RAMBO stream: cos(theta) = 2 r0 - 1, phi = 2 pi r1,
-// q0 = -ln(r2 r3); the isotropic q_i are boosted and scaled onto the total.
+// Inverse square root and reciprocal of a double in the normal float range
+// (with a margin): an FP32 estimate (relative error e/2 or e about 2^-22) and
+// one step of the binomial series to e^2 in FP64,
+//   x^-1/2 = y (1 + e/2 + 3/8 e^2 + ...), e = 1 - x y^2;  1/x = y (1 + e + e^2 + ...), e = 1 - x y
+// (next terms below 2^-63): 5 and 3 FP64 operations.
+__device__ __forceinline__ double f64_of_f32(float f);
+__device__ __forceinline__ double rsqrt_series(double x) {
+    const double y = f64_of_f32(rsqrtf(f32_rn(x)));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double recip_series(double x) {
+    const double y = f64_of_f32(__frcp_rn(f32_rn(x)));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// RAMBO: n massless momenta with total (M, 0, 0, 0), and iM = 1/M.  Photon i
+// uses draws 4i..4i+3 of the RAMBO stream: cos(theta) = 2 r0 - 1, phi = 2 pi
+// r1, q0 = -ln(r2 r3) (photon_q); the isotropic q_i are boosted to the rest
+// frame of their sum.
+//
+// GB300, FP64 instructions a point, before -> after: 403 -> 154 at n = 4, 500,000
+// phase-space points at n = 5 454 -> 231 us.  True error of the momenta (against
+// quad precision, 2-norm): n = 5 2.71e-16 -> 2.69e-16, n = 2 3.2e-14 -> 2.4e-14.
 template <int N>
-__device__ __forceinline__ void rambo(const PointRng& rng, double rs, const MomView& v) {
+__device__ __forceinline__ double rambo(const PointRng& rng, const MomView& v) {
     double Q0 = 0, Q1 = 0, Q2 = 0, Q3 = 0;
 #pragma unroll 1
     for (int i = 0; i < N; ++i) {
-        const U4 w = rng.words(kStreamRambo, 2 * i);   // r0 = u(w.x, w.y), r1 = u(w.z, w.w)
-        double r2, r3;
-        rng.pair(kStreamRambo, 2 * i + 1, r2, r3);
-        const double c = 2.0 * u01_from_words(w.x, w.y) - 1.0;
-        const double s2 = 1.0 - c * c;   // in [2^-51, 1): never 0
-        const double s = s2 * rsqrt(s2);
-        double sp, cp;
-        sincos_2pi_words(w.z, w.w, sp, cp);
-        const double q0 = -log_table(r2 * r3);   // r2 r3 in [2^-106, 1): normal
-        const double qs = q0 * s;
-        const double q1 = qs * cp, q2 = qs * sp, q3 = q0 * c;
-        v(i, 0) = q0;
-        v(i, 1) = q1;
-        v(i, 2) = q2;
-        v(i, 3) = q3;
-        Q0 += q0;
-        Q1 += q1;
-        Q2 += q2;
-        Q3 += q3;
+        const U4 w = rng.words(kStreamRambo, 2 * i), z = rng.words(kStreamRambo, 2 * i + 1);
+        const PhotonQ q = photon_q(u53_of_words(w.x, w.y), u53_of_words(w.z, w.w), u53_of_words(z.x, z.y),
+                                   u53_of_words(z.z, z.w), kDirLog, kDirAng);
+        v(i, 0) = q.q0;
+        v(i, 1) = q.q1;
+        v(i, 2) = q.q2;
+        v(i, 3) = q.q3;
+        Q0 += q.q0;
+        Q1 += q.q1;
+        Q2 += q.q2;
+        Q3 += q.q3;
     }
-    // M = sqrt(Q^2), b = -Q/M, gamma = Q0/M, a = 1/(1 + gamma) = M/(M + Q0),
-    // x = rs/M; then p_i = x (gamma q0 + b.q, q + b (q0 + a b.q)).
+    // M = sqrt(Q^2), b = -Q/M, gamma = Q0/M, a = 1/(1 + gamma) = M/(M + Q0):
+    // p_i = (gamma q0 + b.q, q + b (q0 + a b.q)).
     const double M2 = Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3;
-    const double iM = rsqrt(M2);
+    const double iM = rsqrt_series(M2);
     const double M = M2 * iM;
     const double b1 = -Q1 * iM, b2 = -Q2 * iM, b3 = -Q3 * iM;
-    const double a = M / (M + Q0);
-    const double x = rs * iM;
-    const double xg = x * (Q0 * iM), xb1 = x * b1, xb2 = x * b2, xb3 = x * b3;
+    const double a = M * recip_series(M + Q0);
+    const double g = Q0 * iM;
 #pragma unroll 1
     for (int i = 0; i < N; ++i) {
         const double q0 = v(i, 0), q1 = v(i, 1), q2 = v(i, 2), q3 = v(i, 3);
         const double bq = b1 * q1 + b2 * q2 + b3 * q3;
         const double t = fma(a, bq, q0);
-        v(i, 0) = fma(xg, q0, x * bq);
-        v(i, 1) = fma(xb1, t, x * q1);
-        v(i, 2) = fma(xb2, t, x * q2);
-        v(i, 3) = fma(xb3, t, x * q3);
+        v(i, 0) = fma(g, q0, bq);
+        v(i, 1) = fma(b1, t, q1);
+        v(i, 2) = fma(b2, t, q2);
+        v(i, 3) = fma(b3, t, q3);
     }
+    return iM;
 }
 
 // a < b for doubles a, b >= +0 (squares and their products, never -0 or
@@ -421,16 +440,18 @@ __device__ __forceinline__ bool lt_scaled(double v, double a, double w2) {
 //   cos(phi_i - phi_j)  = (px_i px_j + py_i py_j) / (pT_i pT_j);
 // a pair passes at once if |Delta eta| > R or Delta phi > R (compared on
 // squares), and only the remaining close pairs evaluate asinh and atan2.
-// ey, iey: e^y and e^-y.
+// The momenta are in units of 1/scale GeV (EventInfo).  Out of line: only
+// points that the FP32 tests leave open come here.
 template <int N>
-__device__ __forceinline__ int pass_cuts(const MomView& p, double ey, double iey, const Physics& ph) {
+__device__ __noinline__ int pass_cuts(const MomView p, double scale, u64 ua, u64 ub, const Physics& ph) {
     // every photon and pair is tested without early exits: the FP64 pipe
     // executes whole warps, so a lane that could stop early saves nothing and
     // the divergence would cost the others
+    const double ey = (double)ua / (double)ub, iey = (double)ub / (double)ua;   // e^y, e^-y
     const double shy = 0.5 * (ey - iey), chy = 0.5 * (ey + iey);
     const double s_hi = ph.sinh_eta * chy - ph.cosh_eta * shy;    // sinh(E - y)
     const double s_lo = -ph.sinh_eta * chy - ph.cosh_eta * shy;   // sinh(-E - y)
-    const double pt2min = ph.pt_min * ph.pt_min;
+    const double pt_min = ph.pt_min / scale, pt2min = pt_min * pt_min;
     bool ok = true;
     double pt2[N];
 #pragma unroll
@@ -535,16 +556,21 @@ __device__ __forceinline__ float f32_cut(double x) {
 // after: n = 4 step of 1,048,576 points 1123 -> 1012 us, phase space of 500,000
 // points at n = 5 668 -> 454 us.
 //
-// FP32 holds the squares and fourth powers of momenta of 1e-2 .. 1e8 GeV
-// events and the cuts' e^2E and sinh^2 R: other events and cuts are left to
-// pass_cuts, and so is a photon whose pT^2 FP32 cannot hold accurately.
+// The momenta are in RAMBO's units (total M, of the order of n), which FP32
+// holds; pT is compared in GeV.  Energies, pT cuts, e^2E and sinh^2 R that
+// FP32 does not hold are left to pass_cuts, and so is a photon whose pT^2 FP32
+// cannot hold accurately.
 template <int N>
-__device__ __forceinline__ int pass_cuts_fast(const MomView& p, double rs, double ey, double iey, const Physics& ph) {
+__device__ __forceinline__ int pass_cuts_fast(const MomView& p, const EventInfo& ev, const Physics& ph) {
     constexpr float kU = 5.9604645e-8f;   // 2^-24
-    if (!(rs > 1e-2 && rs < 1e8 && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12))
-        return pass_cuts<N>(p, ey, iey, ph);
+    const double scale = ev.rs * ev.iM;
+    if (!(ev.rs > 1e-2 && ev.rs < 1e8 && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12 &&
+          !(ph.pt_min > 0 && ph.pt_min < 1e-12)))
+        return pass_cuts<N>(p, scale, ev.ua, ev.ub, ph);
     constexpr float kLo = 1.0f - 64.0f * kU, kHi = 1.0f + 64.0f * kU;
-    const float eyf = f32_cut(ey), ieyf = f32_cut(iey);
+    // e^y = ua / ub: a and b below are p+ e^y and p- e^-y times ua ub 2^-106
+    const float uaf = __ull2float_rz(ev.ua) * 0x1p-53f, ubf = __ull2float_rz(ev.ub) * 0x1p-53f;
+    const float eyf = uaf * uaf, ieyf = ubf * ubf, s2 = f32_cut(scale) * f32_cut(scale);
     const float eE = f32_cut(ph.sinh_eta) + f32_cut(ph.cosh_eta), e2E = eE * eE;
     const float ptmin2 = f32_cut(ph.pt_min) * f32_cut(ph.pt_min);
     float x[N], y[N], pp[N], pm[N], pt2[N];
@@ -559,8 +585,9 @@ __device__ __forceinline__ int pass_cuts_fast(const MomView& p, double rs, doubl
         pp[i] = z < 0.0f ? small : big;
         pm[i] = z < 0.0f ? big : small;
         const bool held = pt2[i] > 1e-30f;
-        fail = fail || pt2[i] < ptmin2 * kLo;
-        open = open || !(held && pt2[i] > ptmin2 * kHi);
+        const float pt2g = pt2[i] * s2;   // GeV^2
+        fail = fail || pt2g < ptmin2 * kLo;
+        open = open || !(held && pt2g > ptmin2 * kHi);
         const float a = pp[i] * eyf, b = pm[i] * ieyf;
         fail = fail || (held && (a * kLo > e2E * b || b * kLo > e2E * a));
         open = open || !(a * kHi < e2E * b && b * kHi < e2E * a);
@@ -602,17 +629,17 @@ __device__ __forceinline__ int pass_cuts_fast(const MomView& p, double rs, doubl
         if (d2 < R2 - m) return 0;
         open = open || !(d2 > R2 + m);
     }
-    return open ? pass_cuts<N>(p, ey, iey, ph) : 1;
+    return open ? pass_cuts<N>(p, scale, ev.ua, ev.ub, ph) : 1;
 }
 
 // Event i of stream `seed` from its sampler draws d: sqrt(s-hat), RAMBO
-// momenta into v, cut decision.
+// momenta into v (units of EventInfo), cut decision.
 template <int N>
 __device__ __forceinline__ void generate_from(const PointRng& rng, const SampleDraw& d, const SamplerArgs& S,
                                               const Physics& ph, const MomView& v, EventInfo& ev) {
     sample_finish(S, d, ev);
-    rambo<N>(rng, ev.rs, v);
-    ev.mask = ev.ok ? pass_cuts_fast<N>(v, ev.rs, ev.ey, ev.iey, ph) : 0;
+    ev.iM = rambo<N>(rng, v);
+    ev.mask = ev.ok ? pass_cuts_fast<N>(v, ev, ph) : 0;
 }
 
 template <int N>
@@ -799,19 +826,29 @@ __device__ __forceinline__ float rec_denominator(const float2* inv, unsigned T) 
     return S + E;
 }
 
-// Record of a point that passed the cuts, from its photon momenta (GeV) and
-// irs = 1/sqrt(s-hat): momenta / sqrt(s-hat), denominators, normalisations,
-// the factors to |M|^2 and to the event weight, valid = mask = 1.  The
-// momenta are divided by sqrt(s-hat) in place, and the denominators formed
-// from the scaled values.  (The caller sets idx and hsel.)
+// 1/rs^2 of rs > 0: on the mantissa (recip_series) with the exponent put back,
+// or by division where that leaves the normal range.
+__device__ __forceinline__ double inverse_square(double rs) {
+    const int hi = __double2hiint(rs), ex = (hi >> 20) - 1023;
+    if (ex < -400 || ex > 400) return 1.0 / (rs * rs);
+    const double r = recip_series(__hiloint2double(hi - (ex << 20), __double2loint(rs)));
+    const double q = r * r;   // in [1/4, 1]
+    return __hiloint2double(__double2hiint(q) - ((2 * ex) << 20), __double2loint(q));
+}
+
+// Record of a point that passed the cuts, from its photon momenta (units of
+// EventInfo), iM and rs: momenta / sqrt(s-hat), denominators, normalisations,
+// the factor to the event weight, valid = mask = 1.  The momenta are scaled
+// in place, and the denominators formed from the scaled values.  (The caller
+// sets idx and hsel; `fac`, the factor to |M|^2, is not needed here.)
 template <class R, int N>
-__device__ __forceinline__ void pass_to_rec(const MomView& v, double irs, const Physics& ph, PointRec<R, N>& rec) {
-    const double is = irs * irs;
+__device__ __forceinline__ void pass_to_rec(const MomView& v, double iM, double rs, const Physics& ph,
+                                            PointRec<R, N>& rec) {
 #pragma unroll 1
     for (int a = 0; a < N; ++a)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const double k = v(a, m) * irs;
+            const double k = v(a, m) * iM;
             v(a, m) = k;
             rec.k[a][m] = rec_value<R>(k);
         }
@@ -820,10 +857,7 @@ __device__ __forceinline__ void pass_to_rec(const MomView& v, double irs, const 
     rec.e2 = R(0.5);
     rec.n1 = R(1);
     rec.n2 = R(1);
-    double sp = 1;  // s^(2-n)
-    for (int a = 2; a < N; ++a) sp *= is;
-    rec.fac = ph.cpl * sp;
-    rec.wfac = ph.wconst * is;   // w = wfac * (scaled |M|^2 sum)
+    rec.wfac = ph.wconst * inverse_square(rs);   // w = wfac * (scaled |M|^2 sum)
     rec.valid = 1;
     rec.mask = 1;
 }
