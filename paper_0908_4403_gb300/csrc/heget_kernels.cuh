@@ -7,6 +7,7 @@
 
 #include "heget_reduce.cuh"
 #include "heget_subset.cuh"
+#include "heget_warp.cuh"
 
 namespace heget {
 
@@ -84,7 +85,9 @@ __host__ __device__ constexpr size_t ward_table_bytes() {
 template <class R, int N, int BLOCK, int TAB = kAlgAny, int HB = -1, int G = -1>
 __host__ __device__ constexpr size_t table_bytes() {
     using SH = ShapeSel<R, N, BLOCK, HB, G>;
-    constexpr size_t a = RoundTables<R, N, BLOCK, SH::HB, SH::G>::bytes, b = ward_table_bytes<R, N, BLOCK>();
+    constexpr size_t a = tree_warp_rounds<R, N, SH::HB>() ? WarpTables<R, N, BLOCK / 32>::bytes
+                                                          : RoundTables<R, N, BLOCK, SH::HB, SH::G>::bytes;
+    constexpr size_t b = ward_table_bytes<R, N, BLOCK>();
     constexpr size_t c = MeetTables<R, N, BLOCK>::bytes, kb = KappaTables<R, N, BLOCK>::bytes;
     constexpr size_t ab = a > b ? a : b, ck = c > kb ? c : kb;
     return align16(TAB == kAlgTree ? ab : TAB == kAlgSubset ? c : TAB == kTabSubsetKappa ? ck
@@ -112,7 +115,12 @@ __device__ __forceinline__ void amp_rounds(unsigned char* smem, PointRec<R, N>* 
         if (kappa) kappa_rounds<R, N, BLOCK, BAR>(smem, recs, cnt, mask);
     } else if constexpr (ALG == kAlgTree) {
         using SH = ShapeSel<R, N, BLOCK, HB, G>;
-        amplitude_rounds<R, N, BLOCK, BAR, SH::HB, SH::G>(smem, recs, cnt, mask);
+        if constexpr (tree_warp_rounds<R, N, SH::HB>()) {
+            amplitude_rounds_warps<R, N, BLOCK, BAR>(smem, recs, cnt, mask);
+            if (BAR != 0 && kappa) group_sync<BAR, BLOCK>();   // the bound reuses the warps' tables
+        } else {
+            amplitude_rounds<R, N, BLOCK, BAR, SH::HB, SH::G>(smem, recs, cnt, mask);
+        }
         if (kappa) kappa_rounds<R, N, BLOCK, BAR>(smem, recs, cnt, mask);
     } else if (alg == kAlgSubset) {
         amp_rounds<R, N, BLOCK, BAR, kAlgSubset>(smem, recs, cnt, mask, alg, kappa);
@@ -255,10 +263,14 @@ __device__ __forceinline__ MomView row_view(double* stage, int srow, int c, doub
 
 // Resident blocks per SM an amp2 kernel is compiled for: the FP32 subset
 // recursion from n = 6 keeps three blocks of its 60 KB tables (at most 85
-// registers a thread); elsewhere the compiler's choice.
+// registers a thread); the FP32 tree's warp rounds (n = 4, 5) two, without
+// which the unrolled closures take 175 registers at n = 5; elsewhere the
+// compiler's choice.
 template <class R, int N, int ALG>
 __host__ __device__ constexpr int amp2_min_blocks() {
-    return sizeof(R) == sizeof(float) && ALG == kAlgSubset && N >= 6 ? 3 : 1;
+    return sizeof(R) != sizeof(float) ? 1
+         : ALG == kAlgSubset ? (N >= 6 ? 3 : 1)
+                             : tree_warp_rounds<R, N, 0>() ? 2 : 1;
 }
 
 template <class R, int N, int BLOCK, bool ESC, int ALG>
