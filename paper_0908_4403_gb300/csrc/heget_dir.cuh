@@ -48,22 +48,26 @@ __host__ __device__ __forceinline__ u64 mulhi63(u64 a, u64 b) {
     return (u64)ah * bh + (t >> 32);
 }
 
-__host__ __device__ __forceinline__ int clz128(u64 h, u64 l) { return h ? clz64(h) : 64 + clz64(l); }
-
-// The top 64 bits of (h, l) << sh, 0 < sh < 128.
-__host__ __device__ __forceinline__ u64 shift_top(u64 h, u64 l, int sh) {
-    return sh < 64 ? (h << sh) | (l >> (64 - sh)) : l << (sh - 64);
+// v 2^e rounded to double, v < 2^63, for results in the normal range; neg:
+// with a minus sign.  The conversion is one instruction on the FP64 pipe; an
+// integer one takes 40.  (v | 1 keeps zero out, half a unit of v's last place.)
+__host__ __device__ __forceinline__ double double_of(u64 v, int e, bool neg) {
+    const u64 b = double_bits((double)(long long)(v | 1u)) + ((u64)(long long)e << 52);
+    return bits_double(neg ? b | (1ull << 63) : b);
+}
+// The same for normalised v (2^62 <= v < 2^63), by integer operations (ties away).
+__host__ __device__ __forceinline__ double double_of_normal(u64 v, int e) {
+    const u64 r = (v >> 10) + ((v >> 9) & 1u);             // 2^52 .. 2^53
+    return bits_double(((u64)(e + 62 + 1022) << 52) + r);   // a carry of the rounding moves into the exponent
 }
 
-// v 2^e rounded to double (ties away), for results in the normal range;
-// neg: with a minus sign.
-__host__ __device__ __forceinline__ double double_of(u64 v, int e, bool neg) {
-    if (v == 0) return 0.0;
-    const int lz = clz64(v);
-    v <<= lz;
-    const u64 r = (v >> 11) + ((v >> 10) & 1u);                 // 2^52 .. 2^53
-    const u64 b = ((u64)(e + 63 - lz + 1022) << 52) + r;         // a carry of the rounding moves into the exponent
-    return bits_double(neg ? b | (1ull << 63) : b);
+// The normalising left shift of a 128-bit product (h, l) and its top 64 bits
+// after a shift by sh, 0 < sh < 128.  h = 0 happens once in 2^40 products: a
+// branch of its own keeps its selects out of the common path.
+__host__ __device__ __forceinline__ int clz_product(u64 h, u64 l) { return h ? clz64(h) : 64 + clz64(l); }
+__host__ __device__ __forceinline__ u64 top_product(u64 h, u64 l, int sh) {
+    if (sh >= 64) return l << (sh - 64);
+    return (h << sh) | (l >> (64 - sh));
 }
 
 // The uniform u = (m + 1/2) 2^-52 of two random words (u01_from_words) as the
@@ -79,8 +83,8 @@ __host__ __device__ __forceinline__ u64 u53_of_words(u32 lo, u32 hi) { return ((
 __host__ __device__ __forceinline__ unsigned __int128 neg_log(u64 a, u64 b, const uint4* logtab) {
     const unsigned __int128 P = (unsigned __int128)a * b;
     const u64 ph = (u64)(P >> 64), pl = (u64)P;
-    const int lz = clz128(ph, pl);
-    const u64 M = shift_top(ph, pl, lz);
+    const int lz = clz_product(ph, pl);
+    const u64 M = top_product(ph, pl, lz);
 #ifdef __CUDA_ARCH__
     const uint4 tb = __ldg(logtab + ((M >> 54) & 511u));
 #else
@@ -137,8 +141,8 @@ __host__ __device__ __forceinline__ void quadrant_cos_sin(u64 f, const ulonglong
 __host__ __device__ __forceinline__ u64 sin_theta(u64 a) {
     const unsigned __int128 P = (unsigned __int128)a * ((1ull << 53) - a);
     const u64 ph = (u64)(P >> 64), pl = (u64)P;
-    const int ze = (clz128(ph, pl) - 24) & ~1;
-    const u64 X = shift_top(ph, pl, 24 + ze);                 // x 2^64
+    const int ze = (clz_product(ph, pl) - 24) & ~1;
+    const u64 X = top_product(ph, pl, 24 + ze);                // x 2^64
     const u32 xh = (u32)(X >> 32);
 #ifdef __CUDA_ARCH__
     const float y = rsqrtf(__uint2float_rn(xh) * 0x1p-32f);
@@ -155,6 +159,16 @@ __host__ __device__ __forceinline__ u64 sin_theta(u64 a) {
     return (g + (d << 1) + ((d2 + (d2 >> 1)) >> 3)) >> (ze >> 1);
 }
 
+// A positive V 2^-72, V < 2^80, as m 2^ex with 2^62 <= m < 2^63 (ex returned).
+__host__ __device__ __forceinline__ int normal_of(unsigned __int128 V, u64& m) {
+    const u64 h = (u64)(V >> 16);
+    const u32 l = (u32)V & 0xFFFFu;
+    const int lz = h ? clz64(h) : 64;
+    m = lz < 64 ? ((h << lz) | (lz <= 16 ? (u64)((l << lz) >> 16) : (u64)l << (lz - 16))) >> 1
+                : (u64)l << (clz64((u64)l) - 1);
+    return lz < 64 ? 17 - lz - 72 : 1 - clz64((u64)l) - 72;
+}
+
 // q = q0 (1, sin th cos phi, sin th sin phi, cos th) of one photon from its
 // four uniforms r0 .. r3 as odd integers (u53_of_words).
 struct PhotonQ {
@@ -162,12 +176,8 @@ struct PhotonQ {
 };
 __host__ __device__ __forceinline__ PhotonQ photon_q(u64 r0, u64 r1, u64 r2, u64 r3, const uint4* logtab,
                                                      const ulonglong2* angtab) {
-    const unsigned __int128 V = neg_log(r2, r3, logtab);
-    // q0 = V 2^-72 = m 2^ex with m < 2^63 normalised (V < 2^80: 96 bits hold it)
-    const u64 vh = (u64)(V >> 32);
-    const int lz = clz128(vh, (u64)(u32)V << 32);
-    const u64 m = shift_top(vh, (u64)(u32)V << 32, lz + 0) >> 1;
-    const int ex = 33 - lz - 72;
+    u64 m;
+    const int ex = normal_of(neg_log(r2, r3, logtab), m);   // q0 = m 2^ex
     u64 c, s;
     quadrant_cos_sin(r1 & ((1ull << 51) - 1), angtab, c, s);
     const u32 quad = (u32)(r1 >> 51);
@@ -175,7 +185,7 @@ __host__ __device__ __forceinline__ PhotonQ photon_q(u64 r0, u64 r1, u64 r2, u64
     const u64 st = sin_theta(r0);
     const u64 cp = quad & 1 ? s : c, sp = quad & 1 ? c : s;
     PhotonQ q;
-    q.q0 = double_of(m, ex, false);
+    q.q0 = double_of_normal(m, ex);
     q.q1 = double_of(mulhi63(m, mulhi63(st, cp)), ex + 2, quad == 1 || quad == 2);
     q.q2 = double_of(mulhi63(m, mulhi63(st, sp)), ex + 2, quad >= 2);
     q.q3 = double_of(mulhi63(m, ct << 11), ex + 1, !(r0 >> 52));

@@ -666,28 +666,33 @@ xsec_batch_kernel(const WorkItem* __restrict__ items, int nitems, const BatchReq
 // amplitudes run.  Each block therefore splits into roles that run
 // concurrently:
 //   consumers (ws_consumers(n, alg, esc) threads, the first warps): the amplitude
-//               rounds, and the sampler draws of the stage two ahead;
-//   producers (ws_stage(n, alg) threads, the last warps): one event per
-//               thread per stage from its draws: the FP64 rest (sqrt(s-hat),
-//               RAMBO, cuts, records).
+//               rounds, and without a sampler's warp the sampler draws of the
+//               stage two ahead;
+//   producers (ws_stage(n, alg) threads, the next warps): one event per
+//               thread per stage from its draws: the rest (sqrt(s-hat),
+//               RAMBO, cuts, records);
+//   sampler (one warp, where ws_sampler says so): the draws two stages ahead.
 // The sampler (the toy PDF's rejection loops) is integer and FP32 work whose
 // iteration counts differ from lane to lane; run on the producers it would
-// idle the FP64 pipe, on the consumers it fills their waits.
+// hold them up, on the consumers it costs 53 warp instructions an event, on a
+// warp of its own with a work queue 20.
 // Producers fill a double-buffered ring of ws_stage(n) point records in shared
 // memory; the two roles hand stages over through named barriers
 //   FULL[s]  (bar.arrive by producers, bar.sync by consumers) and
 //   EMPTY[s] (bar.arrive by consumers, bar.sync by producers);
 // the draws of stage k + 2 go into slot s = k & 1 of a second double buffer
-// before the consumers' EMPTY[s] arrival (those of stages 0 and 1 before the
-// roles split),
-// while the consumers' own rounds synchronise on barrier kBarRounds.  Every
+// before the consumers' EMPTY[s] arrival, or between the sampler's barriers
+// kBarDrawEmpty[s] and kBarDrawFull[s] (those of stages 0 and 1 before the roles
+// split), while the consumers' own rounds synchronise on barrier kBarRounds.  Every
 // thread of both roles runs the same number of stages, so each barrier
-// instance collects exactly ws_consumers + ws_stage arrivals.  A block walks tiles
+// instance collects exactly ws_consumers + ws_stage arrivals (the sampler's:
+// ws_stage + 32).  A block walks tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ...; the grid is sized to the resident
 // blocks so that each block pipelines many stages.
 // ---------------------------------------------------------------------------
 constexpr int kBarRounds = 1, kBarFull = 2, kBarEmpty = 4;   // named barrier ids (2,3 / 4,5)
 constexpr int kBarProducers = 6;                              // producers' stage compaction
+constexpr int kBarDrawFull = 12, kBarDrawEmpty = 14;          // sampler's draws of a slot (12,13 / 14,15)
 
 // Consumer threads: 256; 128 for the tree up to n = 4 without the FP32
 // error bound, whose amplitudes are a small share of the block's work (with
@@ -714,6 +719,14 @@ __host__ __device__ constexpr int ws_stage(int n, int alg) {
     return n <= 4 ? 128 : n <= 6 ? 64 : alg == 1 ? 96 : 32;
 }
 
+// Whether a warp of its own draws for the producers (warp_draws over a whole
+// stage).  GB300, one million points (64 K at n = 8), consumers drawing ->
+// sampler's warp: n = 3 519 -> 443 us, n = 4 630 -> 612, subset n = 4 1006 -> 942, n
+// = 8 685 -> 665.  At n = 2 one warp cannot keep up with the producers (309 ->
+// 349), and at n = 5, 6 32 more threads would cost the consumers registers (two
+// blocks of 352 threads leave 93).
+__host__ __device__ constexpr bool ws_sampler(int n, int alg) { return n == 3 || n == 4 || (n >= 7 && alg == 1); }
+
 __device__ __forceinline__ void named_sync(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
@@ -731,6 +744,11 @@ __host__ __device__ constexpr bool tab_has_bound(int tab) { return tab == kTabTr
 template <int N, int ALG, bool ESC>
 __host__ __device__ constexpr int ws_threads() {
     return ws_consumers(N, ALG, ESC) + ws_stage(N, ALG);
+}
+// with the sampler's warp
+template <int N, int ALG, bool ESC>
+__host__ __device__ constexpr int ws_block_threads() {
+    return ws_threads<N, ALG, ESC>() + (ws_sampler(N, ALG) ? 32 : 0);
 }
 template <class R, int N, int ALG, int TAB>
 __host__ __device__ constexpr size_t ws_recs_offset() {
@@ -750,13 +768,15 @@ __host__ __device__ constexpr int ws_min_blocks() {
 }
 
 template <class R, int N, bool ESC, int ALG>
-__global__ void __launch_bounds__(ws_threads<N, ALG, ESC>(), ws_min_blocks<R, N, ALG, table_alg<ALG, ESC>()>())
+__global__ void __launch_bounds__(ws_block_threads<N, ALG, ESC>(), ws_min_blocks<R, N, ALG, table_alg<ALG, ESC>()>())
 xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics ph,
                Partial* __restrict__ partials, double* __restrict__ w_out, EscArgs esc) {
     constexpr int kWsConsumers = ws_consumers(N, ALG, ESC);
     constexpr int kWsStage = ws_stage(N, ALG);
-    constexpr int kWsThreads = ws_threads<N, ALG, ESC>();
-    static_assert(kWsThreads == kWsConsumers + kWsStage, "block shape");
+    constexpr int kRingThreads = ws_threads<N, ALG, ESC>();          // consumers and producers
+    constexpr int kWsThreads = ws_block_threads<N, ALG, ESC>();
+    constexpr bool kSampler = ws_sampler(N, ALG);
+    constexpr int kDrawThreads = kWsStage + 32;   // producers and the sampler's warp
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int TAB = table_alg<ALG, ESC>();
     PointRec<R, N>* ring = reinterpret_cast<PointRec<R, N>*>(smem + ws_recs_offset<R, N, ALG, TAB>());
@@ -776,6 +796,8 @@ xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physi
         for (int p = lid; p < kWsStage; p += nthr)
             if (t0 + p < npts) s_draw[s][p] = sample_draw(S, PointRng(seed, (uint64_t)(i0 + t0 + p)));
     };
+    // the first two stages' draws by all threads: the shortest way to a short
+    // launch's only stage
     for (int k = 0; k < 2 && k < count; ++k) draw_stage(k, k, tid, kWsThreads);
     __syncthreads();
     // the producer owning slot g of stage k folds that point's weight into its
@@ -805,22 +827,37 @@ xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physi
             esc_n += tot;
         }
     };
-    if (tid >= kWsConsumers) {
+    if (kSampler && tid >= kWsConsumers + kWsStage) {
+        // sampler
+        for (int k = 2; k < count; ++k) {
+            const int s = k & 1;
+            named_sync(kBarDrawEmpty + s, kDrawThreads);
+            const long long t0 = stage_t0(k);
+            warp_draws(S, seed, [&](int p) { return (uint64_t)(i0 + t0 + p); },
+                       (int)min((long long)kWsStage, npts - t0), s_draw[s]);
+            __threadfence_block();
+            named_arrive(kBarDrawFull + s, kDrawThreads);
+        }
+    } else if (tid >= kWsConsumers) {
         // producers
         const int g = tid - kWsConsumers;
         const MomView v{stage + g, kWsStage, kMomSlots};
         for (int k = 0; k < count; ++k) {
             const int s = k & 1;
             if (k >= 2) {
-                named_sync(kBarEmpty + s, kWsThreads);
+                named_sync(kBarEmpty + s, kRingThreads);
                 harvest(k - 2, g);
             }
+            if (kSampler && k >= 2) named_sync(kBarDrawFull + s, kDrawThreads);
             const long long t0 = stage_t0(k);
             const int cnt = (int)min((long long)kWsStage, npts - t0);
+            const SampleDraw draw = s_draw[s][g];
+            if constexpr (kSampler)
+                if (k + 2 < count) named_arrive(kBarDrawEmpty + s, kDrawThreads);
             EventInfo ev;
             bool pass = false;
             if (g < cnt) {
-                generate_from<N>(PointRng(seed, (uint64_t)(i0 + t0 + g)), s_draw[s][g], S, ph, v, ev);
+                generate_from<N>(PointRng(seed, (uint64_t)(i0 + t0 + g)), draw, S, ph, v, ev);
                 pass = ev.ok && ev.mask;
                 acc.npass += ev.mask;
                 acc.ntotal += 1;
@@ -855,25 +892,25 @@ xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physi
             named_sync(kBarProducers, kWsStage);
             if (g == 0) stage_n[s] = tot;
             __threadfence_block();
-            named_arrive(kBarFull + s, kWsThreads);
+            named_arrive(kBarFull + s, kRingThreads);
         }
     } else {
         // consumers
         for (int k = 0; k < count; ++k) {
             const int s = k & 1;
-            named_sync(kBarFull + s, kWsThreads);
+            named_sync(kBarFull + s, kRingThreads);
             const int cnt = stage_n[s];
             amp_rounds<R, N, kWsConsumers, kBarRounds, ALG>(smem, ring + s * ring_stride, cnt, nullptr, ph.alg, ESC);
             if (k + 2 < count) {
-                draw_stage(k + 2, s, tid, kWsConsumers);   // the producers read slot s after EMPTY[s]
+                if constexpr (!kSampler) draw_stage(k + 2, s, tid, kWsConsumers);   // the producers read slot s after EMPTY[s]
                 __threadfence_block();
-                named_arrive(kBarEmpty + s, kWsThreads);
+                named_arrive(kBarEmpty + s, kRingThreads);
             }
         }
     }
     __syncthreads();
     // the last (up to) two stages were never reclaimed: harvest them now
-    if (tid >= kWsConsumers) {
+    if (tid >= kWsConsumers && tid < kRingThreads) {
         for (int k = count - 2 < 0 ? 0 : count - 2; k < count; ++k) harvest(k, tid - kWsConsumers);
         if (ESC && tid == kWsConsumers) esc.cnt[blockIdx.x] = min(esc_n, esc.cap);
     }

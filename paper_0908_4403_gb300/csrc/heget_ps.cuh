@@ -100,27 +100,25 @@ __device__ __forceinline__ float u01_estimate(uint32_t hi) {
 // same way; the FP64 test runs only inside that band (about 2e-6 of the
 // tries).
 //
-// The loop itself is integer and FP32 work (plus the rare FP64 tie-break);
-// it returns the accepted try's random words, and the caller converts them to
-// x = u^2 in FP64 after the loop, where the lanes of a warp have converged.
+// Integer and FP32 work (plus the rare FP64 tie-break) on the random words of
+// one block.
+__device__ __forceinline__ bool toy_pdf_accepts(const U4& w) {
+    const float uf = u01_estimate(w.y), vf = u01_estimate(w.w);
+    const float of = 1.0f - uf * uf;
+    const float tf = of * of * of;
+    if (vf < tf - 0x1p-20f) return true;
+    if (vf > tf + 0x1p-20f) return false;
+    const double u = u01_from_words(w.x, w.y), v = u01_from_words(w.z, w.w);
+    const double om = __dsub_rn(1.0, __dmul_rn(u, u));
+    return v < __dmul_rn(__dmul_rn(om, om), om);
+}
+
+// The accepted try's random words (false when the bound of tries is hit).
 __device__ __forceinline__ bool toy_pdf_draw(const PointRng& rng, uint32_t& blk, int max_tries, uint32_t& wx,
                                              uint32_t& wy) {
     for (int t = 0; t < max_tries; ++t) {
-        const U4 w = philox4x32_10(U4{rng.ilo, rng.ihi, blk++, kStreamSqrtS}, rng.k0, rng.k1);
-        const float uf = u01_estimate(w.y), vf = u01_estimate(w.w);
-        const float of = 1.0f - uf * uf;
-        const float tf = of * of * of;
-        bool accept;
-        if (vf < tf - 0x1p-20f) {
-            accept = true;
-        } else if (vf > tf + 0x1p-20f) {
-            accept = false;
-        } else {
-            const double u = u01_from_words(w.x, w.y), v = u01_from_words(w.z, w.w);
-            const double om = __dsub_rn(1.0, __dmul_rn(u, u));
-            accept = v < __dmul_rn(__dmul_rn(om, om), om);
-        }
-        if (accept) {
+        const U4 w = rng.words(kStreamSqrtS, blk++);
+        if (toy_pdf_accepts(w)) {
             wx = w.x;
             wy = w.y;
             return true;
@@ -150,10 +148,11 @@ __device__ __forceinline__ double event_rapidity(const EventInfo& ev) {
     const __int128 d = (__int128)neg_log(ev.ub, 1ull << 53, kDirLog) - (__int128)neg_log(ev.ua, 1ull << 53, kDirLog);
     const bool neg = d < 0;
     const unsigned __int128 a = neg ? -(unsigned __int128)d : (unsigned __int128)d;   // y 2^72, below 2^80
-    const u64 h = (u64)(a >> 32), l = (u64)(u32)a << 32;
-    if ((h | l) == 0) return 0.0;
-    const int lz = clz128(h, l);
-    return double_of(lz ? shift_top(h, l, lz) : h, 32 - lz - 72, neg);
+    if (a == 0) return 0.0;
+    u64 m;
+    const int ex = normal_of(a, m);
+    const double y = double_of_normal(m, ex);
+    return neg ? -y : y;
 }
 
 // Helicity sampling (the paper's events carry one random helicity
@@ -190,6 +189,18 @@ struct alignas(16) SampleDraw {
     __device__ __forceinline__ void set(int tries, int ok) { ax = (ax & ~0xFFFu) | ((uint32_t)tries << 1) | (uint32_t)ok; }
 };
 
+// The floor test r > floor, r = 2 E sqrt(x1 x2) in FP64, of a draw's two
+// fractions: the test u_a u_b > floor / (2 E) on the uniforms behind x = u^2,
+// whose FP32 estimates (within 2^-24) settle it outside a band of +-16 2^-24
+// around the threshold; the FP64 r decides inside it.
+__device__ __forceinline__ bool above_floor(const SamplerArgs& S, const SampleDraw& d) {
+    const float p = u01_estimate(d.ay) * u01_estimate(d.by);
+    if (p > S.band_hi) return true;
+    if (p < S.band_lo) return false;
+    const double a = toy_pdf_x_of(d.ax, d.ay), b = toy_pdf_x_of(d.bx, d.by);   // rare
+    return 2.0 * S.e_beam * sqrt(a * b) > S.floor;
+}
+
 __device__ __forceinline__ SampleDraw sample_draw(const SamplerArgs& S, const PointRng& rng) {
     SampleDraw d{0u, 0u, 0u, 0u};
     if (S.kind == HEGET_SAMPLER_FIXED) {
@@ -203,24 +214,12 @@ __device__ __forceinline__ SampleDraw sample_draw(const SamplerArgs& S, const Po
         d.set(1, 1);
         return d;
     }
-    // The floor test r > floor, r = 2 E sqrt(x1 x2) in FP64, is the test
-    // u_a u_b > floor / (2 E) on the uniforms behind x = u^2; their FP32
-    // estimates (within 2^-24) settle it outside a band of +-16 2^-24 around
-    // the threshold, and the FP64 r decides inside it.  So the loop runs on
-    // integer and FP32 work, and r and the fractions are formed once, by
-    // sample_finish.
     uint32_t blk = 0;
     int tries = S.max_tries, ok = 0;
     for (int t = 1; t <= S.max_tries; ++t) {
         if (!toy_pdf_draw(rng, blk, S.max_tries, d.ax, d.ay)) break;
         if (!toy_pdf_draw(rng, blk, S.max_tries, d.bx, d.by)) break;
-        const float p = u01_estimate(d.ay) * u01_estimate(d.by);
-        bool pass = p > S.band_hi;
-        if (!pass && p >= S.band_lo) {   // rare
-            const double a = toy_pdf_x_of(d.ax, d.ay), b = toy_pdf_x_of(d.bx, d.by);
-            pass = 2.0 * S.e_beam * sqrt(a * b) > S.floor;
-        }
-        if (pass) {
+        if (above_floor(S, d)) {
             tries = t;
             ok = 1;
             break;
@@ -228,6 +227,65 @@ __device__ __forceinline__ SampleDraw sample_draw(const SamplerArgs& S, const Po
     }
     d.set(tries, ok);
     return d;
+}
+
+// The draws (sample_draw) of the cnt events index(0 .. cnt - 1) of a stream
+// into out, by one warp.  The toy PDF's rejection loops take five blocks of
+// random words an event on average and fifteen in the slowest of 32, so a lane
+// that has finished an event takes the next one, and every pass of the loop
+// tests one block in (nearly) every lane: about 28 passes for 128 events
+// instead of 4 x 15, 20 instructions an event instead of 53.  All lanes must
+// call it; the caller synchronises before other warps read out.
+template <class Index>
+__device__ __forceinline__ void warp_draws(const SamplerArgs& S, uint64_t seed, const Index& index, int cnt,
+                                           SampleDraw* out) {
+    const int lane = threadIdx.x & 31;
+    if (S.kind != HEGET_SAMPLER_TOY_PDF) {
+        for (int p = lane; p < cnt; p += 32) out[p] = sample_draw(S, PointRng(seed, index(p)));
+        return;
+    }
+    int e = lane, next = 32;
+    bool active = e < cnt, second = false;
+    uint32_t blk = 0;
+    int t = 1, inner = 0;
+    SampleDraw d{0u, 0u, 0u, 0u};
+    while (__any_sync(0xffffffffu, active)) {
+        bool done = false;
+        if (active) {
+            const U4 w = PointRng(seed, index(e)).words(kStreamSqrtS, blk++);
+            int ok = 0;
+            if (toy_pdf_accepts(w)) {
+                inner = 0;
+                if (!second) {
+                    d.ax = w.x;
+                    d.ay = w.y;
+                } else {
+                    d.bx = w.x;
+                    d.by = w.y;
+                    ok = above_floor(S, d);
+                    done = ok || t == S.max_tries;
+                    t += !ok;
+                }
+                second = !second;
+            } else {
+                done = ++inner == S.max_tries;
+            }
+            if (done) {
+                d.set(ok ? t : S.max_tries, ok);
+                out[e] = d;
+            }
+        }
+        const unsigned fin = __ballot_sync(0xffffffffu, done);
+        if (done) {
+            e = next + __popc(fin & ((1u << lane) - 1u));
+            active = e < cnt;
+            second = false;
+            blk = 0;
+            t = 1;
+            inner = 0;
+        }
+        next += __popc(fin);
+    }
 }
 
 // sqrt(s-hat) and the outer attempts from the draws: 2 E sqrt(x1 x2) = 2 E ua
@@ -244,8 +302,8 @@ __device__ __forceinline__ void sample_finish(const SamplerArgs& S, const Sample
         ev.ua = u53_of_words(d.ax, d.ay);
         ev.ub = u53_of_words(d.bx, d.by);
         const unsigned __int128 P = (unsigned __int128)ev.ua * ev.ub;
-        const int lz = clz128((u64)(P >> 64), (u64)P);
-        ev.rs = 2.0 * S.e_beam * double_of(shift_top((u64)(P >> 64), (u64)P, lz), 64 - lz - 106, false);
+        const int lz = clz_product((u64)(P >> 64), (u64)P);
+        ev.rs = 2.0 * S.e_beam * double_of_normal(top_product((u64)(P >> 64), (u64)P, lz) >> 1, 65 - lz - 106);
     } else {
         ev.rs = S.floor;
     }
@@ -369,7 +427,8 @@ __device__ __forceinline__ double recip_series(double x) {
 // frame of their sum.
 //
 // GB300, FP64 instructions a point, before -> after: 403 -> 154 at n = 4, 500,000
-// phase-space points at n = 5 454 -> 231 us.  True error of the momenta (against
+// phase-space points at n = 5 454 -> 226 us (unrolling the loops by 2 or 4: no
+// gain, more instruction-cache misses).  True error of the momenta (against
 // quad precision, 2-norm): n = 5 2.71e-16 -> 2.69e-16, n = 2 3.2e-14 -> 2.4e-14.
 template <int N>
 __device__ __forceinline__ double rambo(const PointRng& rng, const MomView& v) {
