@@ -1,10 +1,19 @@
 // heget_hist.cu -- kinematic distributions (Sec. 5, Fig. 2): weighted
-// histograms of photon observables of the generated events.  The events are
-// regenerated from the counter-based generator; every block sums each tile's
-// entries per bin in a fixed order and folds the tile sums into double-double
-// bin sums, and the block partials are combined in block order, so results
-// are reproducible bit for bit for a given launch shape (one resident wave,
-// set by the GPU).
+// histograms of photon observables of the generated events.  The events of
+// nonzero weight are regenerated from the counter-based generator, 256 at a
+// time; their bins come from FP32 observables wherever FP32 settles them, and
+// the weights are added as integers (exactly) within a batch and in
+// double-double across batches and blocks, in a fixed order, so results are
+// reproducible bit for bit for a given launch shape (one resident wave, set by
+// the GPU).
+//
+// What bounded the earlier form (GB300, five histograms of 1,048,576 events at
+// n = 4: 5480 us): 2690 FP64 instruction slots an event -- the observables'
+// asinh, atan2, log and square roots in FP64, bin sums with one active lane an
+// FP64 instruction, and the events of zero weight, generated and dropped.
+// Here, 97 slots (41 % of the FP64 pipe), 154 warp instructions an event: 586 us
+// with the finalisation's 88; bound by the barriers between the passes of a
+// batch (five a histogram).
 #include <algorithm>
 #include <cmath>
 
@@ -14,144 +23,347 @@
 namespace heget {
 namespace {
 
-constexpr int kHistBlock = 128;   // points per block tile, one per thread
+constexpr int kHistBlock = 256;   // events of a batch, one per thread
 
 struct HistSpecDev {
     int kind, nbins, off, pad;   // off: first bin of this histogram in the block's bin array
     double lo, scale;            // scale = nbins / (hi - lo), formed on the host
+    float lo_f, scale_f;
 };
 
 struct HistArgs {
     HistSpecDev spec[HEGET_HIST_MAX_SPECS];
-    int nspec, total;
+    int nspec, total, most;   // bins of all histograms, of the largest
 };
 
 // Bin of x: 0 below lo (and NaN), nbins + 1 at or above hi, else
 // 1 + floor((x - lo) scale), in FP64 without contraction.
-__device__ __forceinline__ int hist_bin(double x, const HistSpecDev& h) {
-    if (!(x >= h.lo)) return 0;
-    const double t = __dmul_rn(__dsub_rn(x, h.lo), h.scale);
-    if (t >= (double)h.nbins) return h.nbins + 1;
+__device__ __forceinline__ int hist_bin(double x, int nbins, double lo, double scale) {
+    if (!(x >= lo)) return 0;
+    const double t = __dmul_rn(__dsub_rn(x, lo), scale);
+    if (t >= (double)nbins) return nbins + 1;
     return 1 + (int)t;
+}
+
+constexpr float kHistU = 5.9604645e-8f;   // 2^-24
+
+// The same bin from an FP32 value xf of x, |xf - x| <= err: -1 unless the bin
+// is certain.  (x - lo) scale carries err scale, the roundings of lo and of the
+// difference (4 u |lo|, u |xf|) and 4 u of itself; every bin edge is an integer.
+__device__ __forceinline__ int hist_bin_f(float xf, float err, const HistSpecDev& h) {
+    const float t = (xf - h.lo_f) * h.scale_f;
+    const float d = (err + 4.0f * kHistU * (fabsf(h.lo_f) + fabsf(xf))) * h.scale_f + 4.0f * kHistU * fabsf(t);
+    const float nb = (float)h.nbins;
+    if (t < -d) return 0;
+    if (t > nb + d) return h.nbins + 1;
+    if (fabsf(t - rintf(t)) > d) return t < nb ? 1 + (int)t : -1;
+    return -1;   // next to an edge, or not a number
 }
 
 __host__ __device__ constexpr int hist_entries_max(int n) {
     return n * (n - 1) / 2 > n ? n * (n - 1) / 2 : n;
 }
 
-__host__ __device__ constexpr size_t hist_smem_bytes(int n, int total) {
-    return (size_t)n * kMomSlots * kHistBlock * sizeof(double)   // momenta, then photon observables
-           + 2 * (size_t)total * sizeof(DD)                          // bin sums of w and w^2
-           + 2 * (size_t)kHistBlock * sizeof(double)                 // weights, sqrt(s-hat)
-           + (size_t)hist_entries_max(n) * kHistBlock * sizeof(short);   // bins of the entries
+// Shared memory of a block: momenta; the weights as integers (w, w^2); the
+// entries (bin, place in it) and the events sorted by bin; counts and offsets
+// per bin; bin sums of w and w^2; sampler draws; the list of events.
+struct HistFixed {
+    __int128 w, w2;
+};
+__host__ __device__ constexpr size_t hist_smem_bytes(int n, int total, int most) {
+    return (size_t)n * kMomSlots * kHistBlock * sizeof(double) + kHistBlock * sizeof(HistFixed) +
+           2 * (size_t)total * sizeof(DD) + kHistBlock * sizeof(SampleDraw) +
+           2 * kHistBlock * (sizeof(long long) + sizeof(double)) +
+           (size_t)hist_entries_max(n) * kHistBlock * (sizeof(unsigned) + sizeof(unsigned char)) +
+           2 * (size_t)most * sizeof(unsigned);
 }
 
+// One event's observables in FP64, for the bins that FP32 leaves open.
+struct HistEvent {
+    MomView v;
+    double scale, y;
+    __device__ __forceinline__ double pt(int i) const {
+        const double px = v(i, 1) * scale, py = v(i, 2) * scale;
+        return sqrt(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)));
+    }
+    __device__ __forceinline__ double eta(int i) const { return asinh(v(i, 3) * scale / pt(i)) + y; }
+    __device__ __forceinline__ double dr(int a, int b) const {
+        double dphi = fabs(atan2(v(a, 2) * scale, v(a, 1) * scale) - atan2(v(b, 2) * scale, v(b, 1) * scale));
+        if (dphi > M_PI) dphi = 2.0 * M_PI - dphi;
+        const double deta = eta(a) - eta(b);
+        return sqrt(__dadd_rn(__dmul_rn(deta, deta), __dmul_rn(dphi, dphi)));
+    }
+};
+// Observable `kind` of photon i or pair (i, j) (or the event's extreme) in FP64, binned.
 template <int N>
-__global__ void __launch_bounds__(kHistBlock)
+__device__ __noinline__ int hist_bin_exact(const MomView v, double scale, u64 ua, u64 ub, int i, int j, int kind,
+                                           int nbins, double lo, double per_unit) {
+    EventInfo ev;
+    ev.ua = ua;
+    ev.ub = ub;
+    const HistEvent e{v, scale, ua == ub ? 0.0 : event_rapidity(ev)};
+    double x = 0.0;
+    if (kind == HEGET_OBS_PT) x = e.pt(i);
+    else if (kind == HEGET_OBS_ETA) x = e.eta(i);
+    else if (kind == HEGET_OBS_DR) x = e.dr(i, j);
+    else if (kind == HEGET_OBS_PT_MAX) {
+        x = e.pt(0);
+        for (int a = 1; a < N; ++a) x = e.pt(a) > x ? e.pt(a) : x;
+    } else {
+        x = e.dr(0, 1);
+        for (int a = 0; a < N; ++a)
+            for (int b = a + 1; b < N; ++b) {
+                const double d = e.dr(a, b);
+                x = d < x ? d : x;
+            }
+    }
+    return hist_bin(x, nbins, lo, per_unit);
+}
+
+// (Three blocks an SM up to n = 5: 85 registers.)
+template <int N>
+__global__ void __launch_bounds__(kHistBlock, N <= 5 ? 3 : 1)
 hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics ph,
             const double* __restrict__ w, HistArgs H, double* __restrict__ parts) {
-    constexpr int NP = N * (N - 1) / 2;
+    constexpr int NP = N * (N - 1) / 2, NW = kHistBlock / 32;
     constexpr int E = hist_entries_max(N);
+    // w: terms below 2^(53 + kTop); w^2: products of mantissas below 2^(106 + kTop2); a bin has at most
+    // E kHistBlock < 2^13 terms of a batch
+    constexpr int kTop = 60, kTop2 = 7, kSpan = 30;
     extern __shared__ __align__(16) unsigned char smem[];
-    double* stage = reinterpret_cast<double*>(smem);
-    DD* hw = reinterpret_cast<DD*>(stage + (size_t)N * kMomSlots * kHistBlock);
+    HistFixed* fx = reinterpret_cast<HistFixed*>(smem);
+    SampleDraw* draws = reinterpret_cast<SampleDraw*>(fx + kHistBlock);
+    DD* hw = reinterpret_cast<DD*>(draws + kHistBlock);
     DD* hw2 = hw + H.total;
-    double* wt = reinterpret_cast<double*>(hw2 + H.total);
-    double* rs = wt + kHistBlock;
-    short* bins = reinterpret_cast<short*>(rs + kHistBlock);   // [entry][point]
-    const int tid = threadIdx.x;
+    double* stage = reinterpret_cast<double*>(hw2 + H.total);
+    long long* list = reinterpret_cast<long long*>(stage + (size_t)N * kMomSlots * kHistBlock);   // events to come
+    double* lw = reinterpret_cast<double*>(list + 2 * kHistBlock);                                // their weights
+    unsigned* ent = reinterpret_cast<unsigned*>(lw + 2 * kHistBlock);   // [entry][event]: bin | place << 10
+    unsigned* cnt = ent + E * kHistBlock;
+    unsigned* off = cnt + H.most;
+    unsigned char* sorted = reinterpret_cast<unsigned char*>(off + H.most);
+    HistFixed* bin_sum = reinterpret_cast<HistFixed*>(draws);
+    __shared__ int s_cnt[NW];
+    __shared__ unsigned s_em[NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int b = tid; b < H.total; b += kHistBlock) hw[b] = hw2[b] = DD{0.0, 0.0};
     const MomView v{stage + tid, kHistBlock, kMomSlots};
-    for (long long t0 = (long long)blockIdx.x * kHistBlock; t0 < npts; t0 += (long long)gridDim.x * kHistBlock) {
-        const int cnt = (int)min((long long)kHistBlock, npts - t0);
-        wt[tid] = 0.0;
-        if (tid < cnt) {
-            EventInfo ev;
-            generate_event<N>(seed, (uint64_t)(i0 + t0 + tid), S, ph, v, ev);
-            const double y = (S.kind == HEGET_SAMPLER_TOY_PDF && ev.ok) ? event_rapidity(ev) : 0.0;
-            const double scale = ev.rs * ev.iM;
-            // the photon observables replace the momenta in the point's column:
-            // slot 0 pT, 1 eta (lab), 2 phi
-#pragma unroll 1
-            for (int i = 0; i < N; ++i) {
-                const double px = v(i, 1) * scale, py = v(i, 2) * scale, pz = v(i, 3) * scale;
-                const double pt = sqrt(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)));
-                v(i, 0) = pt;
-                v(i, 1) = asinh(pz / pt) + y;
-                v(i, 2) = atan2(py, px);
+    long long t0 = (long long)blockIdx.x * kHistBlock;
+    int ln = 0;   // events in the list
+    while (t0 < npts || ln > 0) {
+        // the next events of nonzero weight, in order (a zero weight adds nothing)
+        while (ln < kHistBlock && t0 < npts) {
+            const long long i = t0 + tid;
+            const double wi = i < npts ? w[i] : 0.0;
+            int tot;
+            const int pos = compact_pos<kHistBlock>(wi != 0.0, tid, s_cnt, 0, tot);
+            if (wi != 0.0) {
+                list[ln + pos] = i0 + i;
+                lw[ln + pos] = wi;
             }
-            wt[tid] = w[t0 + tid];
-            rs[tid] = ev.rs;
+            ln += tot;
+            t0 += (long long)gridDim.x * kHistBlock;
         }
-        for (int s = 0; s < H.nspec; ++s) {
-            const HistSpecDev& h = H.spec[s];
-            int m = 0;
-            if (tid < cnt && wt[tid] != 0.0) {   // a zero weight adds nothing
-                switch (h.kind) {
-                    case HEGET_OBS_PT_MAX: {
-                        double x = v(0, 0);
-                        for (int i = 1; i < N; ++i) x = v(i, 0) > x ? v(i, 0) : x;
-                        bins[tid] = (short)hist_bin(x, h);
-                        m = 1;
-                        break;
-                    }
-                    case HEGET_OBS_PT:
-                    case HEGET_OBS_ETA: {
-                        const int slot = h.kind == HEGET_OBS_PT ? 0 : 1;
-                        for (int i = 0; i < N; ++i) bins[i * kHistBlock + tid] = (short)hist_bin(v(i, slot), h);
-                        m = N;
-                        break;
-                    }
-                    case HEGET_OBS_DR:
-                    case HEGET_OBS_DR_MIN: {
-                        double dmin = 0.0;
+        __syncthreads();
+        const int cur = min(ln, kHistBlock);
+        // sampler draws by two warps, 128 events each
+        if (warp < 2 && cur > warp * (kHistBlock / 2)) {
+            const int b0 = warp * (kHistBlock / 2);
+            warp_draws(S, seed, [&](int p) { return (uint64_t)list[b0 + p]; }, min(cur - b0, kHistBlock / 2), draws + b0);
+        }
+        __syncthreads();
+        EventInfo ev;
+        ev.ua = ev.ub = 1;
+        ev.rs = 0.0;
+        double wi = 0.0, scale = 0.0;
+        float pt[N], eta[N], phi[N], yf = 0.0f;
+        bool fp32 = false;   // FP32 holds the event
+        if (tid < cur) {
+            sample_finish(S, draws[tid], ev);
+            scale = ev.rs * rambo<N>(PointRng(seed, (uint64_t)list[tid]), v);
+            wi = lw[tid];
+            fp32 = ev.rs > 1e-2 && ev.rs < 1e8;
+            const float sf = f32_cut(fp32 ? scale : 0.0);
+            // errors (u = 2^-24, components 2 u): pT 10 u; eta = ln((E + |pz|) / pT) 16 u absolute and 2 u of
+            // itself; phi 16 u absolute; y = ln(ua / ub) 10 u absolute and 2 u of itself
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const float e = f32_cut(v(i, 0)), x = f32_cut(v(i, 1)), y = f32_cut(v(i, 2)), z = f32_cut(v(i, 3));
+                const float p2 = x * x + y * y, rp = rsqrtf(p2);
+                pt[i] = p2 * rp * sf;
+                eta[i] = copysignf(logf((e + fabsf(z)) * rp), z);
+                phi[i] = atan2f(y, x);
+                fp32 = fp32 && p2 > 1e-30f;
+            }
+            if (ev.ua != ev.ub) yf = logf(__fdividef(__ull2float_rn(ev.ua), __ull2float_rn(ev.ub)));
+        }
+        // the rest of the list moves up
+        long long keep_i = 0;
+        double keep_w = 0.0;
+        if (cur + tid < ln) {
+            keep_i = list[cur + tid];
+            keep_w = lw[cur + tid];
+        }
+        __syncthreads();
+        if (cur + tid < ln) {
+            list[tid] = keep_i;
+            lw[tid] = keep_w;
+        }
+        ln -= cur;
+        // passes over the batch: the events whose weights lie within 2^kSpan of the largest left, as integers
+        // aligned to it (almost always all of them); infinite and NaN weights make their bins NaN
+        bool left = tid < cur;
+        for (;;) {
+            const int ef = left ? exponent_field(wi) : 0;
+            const unsigned wm = __reduce_max_sync(0xffffffffu, (unsigned)ef);
+            if (lane == 0) s_em[warp] = wm;
+            __syncthreads();
+            int em = 0;
+#pragma unroll
+            for (int q = 0; q < NW; ++q) em = max(em, (int)s_em[q]);
+            if (em == 0) break;
+            const bool mine = left && (em >= 0x7FF ? ef == em : ef >= em - kSpan);
+            left = left && !mine;
+            if (mine && em < 0x7FF) {
+                const u64 u = double_bits(wi);
+                const int f = (int)(u >> 52) & 0x7FF;
+                const u64 m = (u & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull);
+                const unsigned __int128 m2 = (unsigned __int128)m * m;
+                const int sh = kTop2 - 2 * (em - ef);
+                fx[tid].w = fixed_of(wi, em, kTop);
+                fx[tid].w2 = (__int128)(sh >= 0 ? m2 << sh : m2 >> -sh);
+            }
+            for (int s = 0; s < H.nspec; ++s) {
+                const HistSpecDev& h = H.spec[s];
+                const int nb = h.nbins + 2;
+                for (int b = tid; b < nb; b += kHistBlock) cnt[b] = 0;
+                __syncthreads();   // (also: the integers above, s_em read)
+                int m = 0;
+                if (mine) {
+                    auto put = [&](int bin) {
+                        ent[m * kHistBlock + tid] = (unsigned)bin | (atomicAdd(cnt + bin, 1u) << 10);
+                        ++m;
+                    };
+                    auto exact = [&](int i, int j) { 
+                        return hist_bin_exact<N>(v, scale, ev.ua, ev.ub, i, j, h.kind, h.nbins, h.lo, h.scale);
+                    };
+                    if (h.kind == HEGET_OBS_PT_MAX || h.kind == HEGET_OBS_PT) {
+                        float mx = pt[0];
+#pragma unroll
+                        for (int i = 0; i < N; ++i) {
+                            mx = fmaxf(mx, pt[i]);
+                            if (h.kind == HEGET_OBS_PT) {
+                                const int b = fp32 ? hist_bin_f(pt[i], 12.0f * kHistU * pt[i], h) : -1;
+                                put(b >= 0 ? b : exact(i, 0));
+                            }
+                        }
+                        if (h.kind == HEGET_OBS_PT_MAX) {
+                            const int b = fp32 ? hist_bin_f(mx, 12.0f * kHistU * mx, h) : -1;
+                            put(b >= 0 ? b : exact(0, 0));
+                        }
+                    } else if (h.kind == HEGET_OBS_ETA) {
+#pragma unroll
+                        for (int i = 0; i < N; ++i) {
+                            const float x = eta[i] + yf;
+                            const int b =
+                                fp32 ? hist_bin_f(x, kHistU * (32.0f + 4.0f * (fabsf(eta[i]) + fabsf(yf))), h) : -1;
+                            put(b >= 0 ? b : exact(i, 0));
+                        }
+                    } else if (h.kind == HEGET_OBS_DR || h.kind == HEGET_OBS_DR_MIN) {
+                        float dmin = 3.0e38f, emin = 0.0f;   // smallest Delta R, largest error
+#pragma unroll
                         for (int a = 0; a < N; ++a)
+#pragma unroll
                             for (int b = a + 1; b < N; ++b) {
-                                double dphi = fabs(v(a, 2) - v(b, 2));
-                                if (dphi > M_PI) dphi = 2.0 * M_PI - dphi;
-                                const double deta = v(a, 1) - v(b, 1);
-                                const double dr = sqrt(__dadd_rn(__dmul_rn(deta, deta), __dmul_rn(dphi, dphi)));
-                                if (h.kind == HEGET_OBS_DR) bins[m * kHistBlock + tid] = (short)hist_bin(dr, h);
-                                dmin = (m == 0 || dr < dmin) ? dr : dmin;
-                                ++m;
+                                float dphi = fabsf(phi[a] - phi[b]);
+                                if (dphi > 3.14159265f) dphi = 6.28318531f - dphi;
+                                const float deta = eta[a] - eta[b];
+                                const float dr = sqrtf(deta * deta + dphi * dphi);
+                                const float err = kHistU * (80.0f + 4.0f * (fabsf(eta[a]) + fabsf(eta[b])));
+                                if (h.kind == HEGET_OBS_DR) {
+                                    const int q = fp32 ? hist_bin_f(dr, err, h) : -1;
+                                    put(q >= 0 ? q : exact(a, b));
+                                }
+                                dmin = fminf(dmin, dr);
+                                emin = fmaxf(emin, err);
                             }
                         if (h.kind == HEGET_OBS_DR_MIN) {
-                            bins[tid] = (short)hist_bin(dmin, h);
-                            m = 1;
+                            const int q = fp32 ? hist_bin_f(dmin, emin, h) : -1;
+                            put(q >= 0 ? q : exact(0, 1));
                         }
-                        break;
+                    } else {
+                        put(hist_bin(ev.rs, h.nbins, h.lo, h.scale));
                     }
-                    default:
-                        bins[tid] = (short)hist_bin(rs[tid], h);
-                        m = 1;
-                        break;
                 }
-            }
-            for (int e = m; e < E; ++e) bins[e * kHistBlock + tid] = -1;
-            __syncthreads();
-            // thread b folds bin b (and b + kHistBlock, ...) of this histogram:
-            // the tile's points in order, each point's entries in order, into
-            // a plain FP64 tile sum, which joins the block's double-double sum
-            // once per tile.  (An FP64 instruction occupies the pipe for a whole
-            // warp even when one lane runs it, and a match is one lane's work:
-            // two FP64 operations per match instead of a double-double update.)
-            const int ne = h.kind == HEGET_OBS_PT || h.kind == HEGET_OBS_ETA ? N : h.kind == HEGET_OBS_DR ? NP : 1;
-            for (int b = tid; b < h.nbins + 2; b += kHistBlock) {
-                double t1 = 0.0, t2 = 0.0;
-                for (int p = 0; p < cnt; ++p) {
-                    const double wp = wt[p];
-                    if (wp == 0.0) continue;
-                    for (int e = 0; e < ne; ++e)
-                        if (bins[e * kHistBlock + p] == b) {
-                            t1 += wp;
-                            t2 = fma(wp, wp, t2);
+                __syncthreads();
+                // offsets of the bins in the sorted list
+                if (warp == 0) {
+                    unsigned run = 0;
+                    for (int b0 = 0; b0 < nb; b0 += 32) {
+                        const unsigned c = b0 + lane < nb ? cnt[b0 + lane] : 0u;
+                        unsigned x = c;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+                            if (lane >= o) x += y;
                         }
+                        if (b0 + lane < nb) off[b0 + lane] = run + x - c;
+                        run += __shfl_sync(0xffffffffu, x, 31);
+                    }
                 }
-                hw[h.off + b] = dd_add_d(hw[h.off + b], t1);
-                hw2[h.off + b] = dd_add_d(hw2[h.off + b], t2);
+                __syncthreads();
+                for (int e = 0; e < m; ++e) {
+                    const unsigned q = ent[e * kHistBlock + tid];
+                    sorted[off[q & 1023u] + (q >> 10)] = (unsigned char)tid;
+                }
+                __syncthreads();
+                // bin sums: the order of a bin's events is that of the counting, but integer sums do not depend
+                // on it; 2^ls lanes share a bin
+                int ls = 0;
+                while (ls < 5 && (nb << (ls + 1)) <= kHistBlock) ++ls;
+                for (int q0 = 0; q0 < (nb << ls); q0 += kHistBlock) {
+                    const int b = (q0 + tid) >> ls, part = tid & ((1 << ls) - 1);
+                    __int128 a = 0, a2 = 0;
+                    unsigned c = 0;
+                    if (b < nb) {
+                        c = cnt[b];
+                        const unsigned char* o = sorted + off[b];
+                        if (em < 0x7FF)
+                            for (unsigned q = part; q < c; q += 1u << ls) {
+                                a += fx[o[q]].w;
+                                a2 += fx[o[q]].w2;
+                            }
+                    }
+                    for (int o = (1 << ls) >> 1; o > 0; o >>= 1) {
+                        a += shfl_down128(a, o);
+                        a2 += shfl_down128(a2, o);
+                    }
+                    // the sums go to one thread a bin, so that the FP64 additions below run with whole warps (the
+                    // room of the sampler draws: at most 128 bins are shared)
+                    if (ls > 0) {
+                        if (part == 0 && b < nb) bin_sum[b] = HistFixed{a, a2};
+                        __syncthreads();
+                        if (tid < nb) {
+                            a = bin_sum[tid].w;
+                            a2 = bin_sum[tid].w2;
+                            c = cnt[tid];
+                        }
+                    }
+                    const int mb = ls > 0 ? tid : b;
+                    if (mb < nb && c > 0) {
+                        DD *d = hw + h.off + mb, *d2 = hw2 + h.off + mb;
+                        if (em < 0x7FF) {
+                            *d = dd_add(*d, dd_of_int(a, em - 1075 - kTop));
+                            *d2 = dd_add(*d2, dd_of_int(a2, 2 * (em - 1075) - kTop2));
+                        } else {
+                            *d = *d2 = DD{bits_double(0x7FF8000000000000ull), 0.0};
+                        }
+                    }
+                }
+                __syncthreads();
             }
-            __syncthreads();
         }
+        __syncthreads();   // the momenta and s_em are free again
     }
     __syncthreads();
     for (int b = tid; b < H.total; b += kHistBlock) {
@@ -163,45 +375,35 @@ hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics 
     }
 }
 
-// Block partials combined in block order, in two stages so that many
-// threads share the work: stage 1 folds groups of kHistGroup consecutive
-// blocks (bin-major threads), stage 2 the groups of each bin in order into
-// out[2b], out[2b + 1].
-constexpr int kHistGroup = 32;
-
-__global__ void __launch_bounds__(128) hist_group_kernel(const double* __restrict__ parts, int nblocks, int total,
-                                                         double* __restrict__ groups) {
-    const int ngroups = (nblocks + kHistGroup - 1) / kHistGroup;
-    const long long items = (long long)ngroups * total;
-    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-         it += (long long)gridDim.x * blockDim.x) {
-        const int g = (int)(it / total), b = (int)(it - (long long)g * total);
-        DD a{0.0, 0.0}, a2{0.0, 0.0};
-        const int k1 = min(nblocks, (g + 1) * kHistGroup);
-        for (int k = g * kHistGroup; k < k1; ++k) {
-            const double* o = parts + ((size_t)k * total + b) * 4;
-            a = dd_add(a, DD{o[0], o[1]});
-            a2 = dd_add(a2, DD{o[2], o[3]});
-        }
-        double* q = groups + ((size_t)g * total + b) * 4;
-        q[0] = a.hi;
-        q[1] = a.lo;
-        q[2] = a2.hi;
-        q[3] = a2.lo;
+// Block partials of a bin combined by one warp, as integers aligned to the
+// largest exponent (heget_reduce.cuh), into out[2b], out[2b + 1].  (GB300, 608
+// blocks, 234 bins: 57 us as two kernels of double-double additions.)
+__global__ void __launch_bounds__(256) hist_finalize_kernel(const double* __restrict__ parts, int nblocks, int total,
+                                                            double* __restrict__ out) {
+    const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= total) return;
+    int em[2] = {1, 1};
+    for (int k = lane; k < nblocks; k += 32) {
+        const double* o = parts + ((size_t)k * total + b) * 4;
+        em[0] = max(em[0], exponent_field(DD{o[0], o[1]}));
+        em[1] = max(em[1], exponent_field(DD{o[2], o[3]}));
     }
-}
-
-__global__ void __launch_bounds__(128) hist_finalize_kernel(const double* __restrict__ groups, int ngroups,
-                                                            int total, double* __restrict__ out) {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < total; b += gridDim.x * blockDim.x) {
-        DD a{0.0, 0.0}, a2{0.0, 0.0};
-        for (int g = 0; g < ngroups; ++g) {
-            const double* o = groups + ((size_t)g * total + b) * 4;
-            a = dd_add(a, DD{o[0], o[1]});
-            a2 = dd_add(a2, DD{o[2], o[3]});
+    const int top = 73 - (32 - __clz(2 * nblocks));   // 2 nblocks terms below 2^(53 + top)
+    __int128 v[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) em[q] = (int)__reduce_max_sync(0xffffffffu, (unsigned)em[q]);
+    for (int k = lane; k < nblocks; k += 32) {
+        const double* o = parts + ((size_t)k * total + b) * 4;
+        v[0] += fixed_of(DD{o[0], o[1]}, em[0], top);
+        v[1] += fixed_of(DD{o[2], o[3]}, em[1], top);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        for (int o = 16; o > 0; o >>= 1) v[q] += shfl_down128(v[q], o);
+        if (lane == 0) {
+            const DD d = dd_of_fixed(v[q], em[q], top);
+            out[2 * b + q] = d.hi + d.lo;
         }
-        out[2 * b] = a.hi + a.lo;
-        out[2 * b + 1] = a2.hi + a2.lo;
     }
 }
 
@@ -209,7 +411,7 @@ template <int N>
 int launch_hist_n(uint64_t seed, long long i0, long long npts, const SamplerArgs& S, const Physics& ph,
                   const double* w, const HistArgs& H, double* parts, int grid, cudaStream_t st) {
     auto k = hist_kernel<N>;
-    const size_t smem = hist_smem_bytes(N, H.total);
+    const size_t smem = hist_smem_bytes(N, H.total, H.most);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     k<<<grid, kHistBlock, smem, st>>>(seed, i0, npts, S, ph, w, H, parts);
@@ -217,9 +419,9 @@ int launch_hist_n(uint64_t seed, long long i0, long long npts, const SamplerArgs
 }
 
 template <int N>
-int occupancy_hist_n(int total, int* bpsm) {
+int occupancy_hist_n(int total, int most, int* bpsm) {
     auto k = hist_kernel<N>;
-    const size_t smem = hist_smem_bytes(N, total);
+    const size_t smem = hist_smem_bytes(N, total, most);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, k, kHistBlock, smem);
@@ -257,7 +459,10 @@ int heget_hist(heget_ctx* ctx, int n, uint64_t seed, int64_t i0, int64_t N, cons
         H.spec[s].off = total;
         H.spec[s].lo = q.lo;
         H.spec[s].scale = (double)q.nbins / (q.hi - q.lo);
+        H.spec[s].lo_f = (float)H.spec[s].lo;
+        H.spec[s].scale_f = (float)H.spec[s].scale;
         total += q.nbins + 2;
+        H.most = std::max(H.most, q.nbins + 2);
     }
     if (total > HEGET_HIST_MAX_BINS) return fail(HEGET_EINVAL, "%d bins in all; at most %d", total, HEGET_HIST_MAX_BINS);
     H.total = total;
@@ -270,7 +475,7 @@ int heget_hist(heget_ctx* ctx, int n, uint64_t seed, int64_t i0, int64_t N, cons
         return e == cudaSuccess ? HEGET_OK : cuda_fail(e, "heget_hist");
     }
     int bpsm = 0;
-#define OCC(NN) occupancy_hist_n<NN>(total, &bpsm)
+#define OCC(NN) occupancy_hist_n<NN>(total, H.most, &bpsm)
     switch (n) {
         case 2: r = OCC(2); break;
         case 3: r = OCC(3); break;
@@ -282,17 +487,12 @@ int heget_hist(heget_ctx* ctx, int n, uint64_t seed, int64_t i0, int64_t N, cons
     }
 #undef OCC
     if (r) return cuda_fail((cudaError_t)r, "hist occupancy");
-    // one resident wave of at most four blocks per SM (16 warps: enough to
-    // keep the FP64 pipe busy) keeps the block partials few
+    // one resident wave of at most four blocks per SM keeps the block partials few
     const long long tiles = (N + kHistBlock - 1) / kHistBlock;
     const long long wave = (long long)ctx->num_sms * std::min(std::max(bpsm, 1), 4);
     const int grid = (int)std::min(tiles, wave);
-    const int ngroups = (grid + kHistGroup - 1) / kHistGroup;
     const size_t part_bytes = (size_t)grid * total * 4 * sizeof(double);
-    if ((r = grow((void**)&ctx->hist_parts, &ctx->hist_parts_cap,
-                  part_bytes + (size_t)ngroups * total * 4 * sizeof(double), false)))
-        return r;
-    double* groups = ctx->hist_parts + (size_t)grid * total * 4;
+    if ((r = grow((void**)&ctx->hist_parts, &ctx->hist_parts_cap, part_bytes, false))) return r;
     const SamplerArgs S = sampler_args(smp);
     const Physics ph = physics_of(ctx, n);
 #define RUN(NN) launch_hist_n<NN>(seed, i0, N, S, ph, w, H, ctx->hist_parts, grid, st)
@@ -307,13 +507,8 @@ int heget_hist(heget_ctx* ctx, int n, uint64_t seed, int64_t i0, int64_t N, cons
     }
 #undef RUN
     if (r) return cuda_fail((cudaError_t)r, "hist_kernel");
-    const long long items = (long long)ngroups * total;
-    hist_group_kernel<<<(int)std::min<long long>((items + 127) / 128, 4096), 128, 0, st>>>(ctx->hist_parts, grid,
-                                                                                       total, groups);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "hist_group_kernel");
-    hist_finalize_kernel<<<(total + 127) / 128, 128, 0, st>>>(groups, ngroups, total, out);
-    e = cudaGetLastError();
+    hist_finalize_kernel<<<(total + 7) / 8, 256, 0, st>>>(ctx->hist_parts, grid, total, out);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "hist_finalize_kernel");
     return HEGET_OK;
 }

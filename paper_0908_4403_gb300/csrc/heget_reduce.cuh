@@ -91,21 +91,24 @@ __host__ __device__ __forceinline__ double scaled_int(unsigned long long m, int 
     return scalbn((double)m, e);
 }
 
-// The double-double of v 2^(em - 1075 - top), the top 106 bits of v.  em is
-// 0x7FF when a term was not finite: the sum is then NaN, as a double-double
-// sum of such terms is.
-__host__ __device__ __forceinline__ DD dd_of_fixed(__int128 v, int em, int top) {
-    if (em >= 0x7FF) return DD{bits_double(0x7FF8000000000000ull), 0.0};
+// The double-double of v 2^e, the top 106 bits of v.
+__host__ __device__ __forceinline__ DD dd_of_int(__int128 v, int e) {
     const bool neg = v < 0;
     unsigned __int128 u = neg ? -(unsigned __int128)v : (unsigned __int128)v;
     if (u == 0) return DD{0.0, 0.0};
     const unsigned long long uh = (unsigned long long)(u >> 64);
     const int lz = uh ? clz64(uh) : 64 + clz64((unsigned long long)u);
-    u <<= lz;                                   // leading bit at 127
-    const int e = em - 1075 - top - lz;         // weight of bit 0 of u
-    const double hi = scaled_int((unsigned long long)(u >> 75), e + 75);
-    const double lo = scaled_int((unsigned long long)(u >> 22) & ((1ull << 53) - 1), e + 22);
+    u <<= lz;                                   // leading bit at 127, weight of bit 0: 2^(e - lz)
+    const double hi = scaled_int((unsigned long long)(u >> 75), e - lz + 75);
+    const double lo = scaled_int((unsigned long long)(u >> 22) & ((1ull << 53) - 1), e - lz + 22);
     return neg ? DD{-hi, -lo} : DD{hi, lo};
+}
+
+// The double-double of v 2^(em - 1075 - top).  em is 0x7FF when a term was not
+// finite: the sum is then NaN, as a double-double sum of such terms is.
+__host__ __device__ __forceinline__ DD dd_of_fixed(__int128 v, int em, int top) {
+    if (em >= 0x7FF) return DD{bits_double(0x7FF8000000000000ull), 0.0};
+    return dd_of_int(v, em - 1075 - top);
 }
 
 constexpr int kWarpTop = 66;   // 64 terms a warp (hi and lo of 32 lanes), one bit to spare
