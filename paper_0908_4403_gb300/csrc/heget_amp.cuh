@@ -82,10 +82,20 @@ __device__ __forceinline__ void group_sync() {
 
 template <class R> __device__ __forceinline__ R recip(R x);
 template <> __device__ __forceinline__ float recip<float>(float x) { return __frcp_rn(x); }
-template <> __device__ __forceinline__ double recip<double>(double x) { return 1.0 / x; }
+// (the series of heget_ps.cuh inside the FP32 range with a wide margin: 3 and 5
+// FP64 instructions instead of about 10 each)
+__device__ __forceinline__ bool in_series_range(double x) {
+    const int e = (__double2hiint(x) >> 20) & 0x7FF;
+    return e > 1023 - 100 && e < 1023 + 100;
+}
+template <> __device__ __forceinline__ double recip<double>(double x) {
+    return in_series_range(x) ? recip_series(x) : 1.0 / x;
+}
 template <class R> __device__ __forceinline__ R rsq(R x);
 template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
+template <> __device__ __forceinline__ double rsq<double>(double x) {
+    return in_series_range(x) ? rsqrt_series(x) : rsqrt(x);
+}
 
 template <class R> __device__ __forceinline__ R fmad(R a, R b, R c);
 template <> __device__ __forceinline__ float fmad<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }

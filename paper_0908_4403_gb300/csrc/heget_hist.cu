@@ -11,9 +11,8 @@
 // n = 4: 5480 us): 2690 FP64 instruction slots an event -- the observables'
 // asinh, atan2, log and square roots in FP64, bin sums with one active lane an
 // FP64 instruction, and the events of zero weight, generated and dropped.
-// Here, 97 slots (41 % of the FP64 pipe), 154 warp instructions an event: 586 us
-// with the finalisation's 88; bound by the barriers between the passes of a
-// batch (five a histogram).
+// Here, 97 slots (41 % of the FP64 pipe) and 154 warp instructions an event: 532
+// us, bound by the barriers between the passes of a batch (six a histogram).
 #include <algorithm>
 #include <cmath>
 

@@ -17,7 +17,8 @@
 // GB300, warp instructions a point and time, walk -> here: the n = 4 step of
 // 1,048,576 points 661 -> 384 and 1027 -> 644 us (its consumers were what the FP64
 // producers waited for); heget_amp2 of 50,001 rows at n = 5 5013 -> 2500 and 322 ->
-// 190 us; FP64 at n = 4, 262,144 points 3030 -> 2346 us.  What bounds it now: fixed
+// 190 us; FP64 at n = 4, 262,144 points 3030 -> 2346 us, and 1806 with the orders
+// of a pair added first (warp_add_orders).  What bounds it now: fixed
 // latencies and the instruction cache (issue 51 %, FMA pipe 31 %, FP64 pipe 47 %
 // of the fused n = 4 kernel).
 #pragma once
@@ -213,6 +214,26 @@ __device__ __forceinline__ void warp_triples(const WarpTables<R, N, WARPS>& tb, 
     }
 }
 
+// FP64: the rows of the two orders of a photon pair and the pair columns of
+// the two orders of the pair left are added first (distributivity), so that a
+// set of two photons closes once instead of four times: 48 multiply-adds a
+// lane at n = 4 instead of 192, where the FP64 pipe is what bounds the rounds.
+// (FP32 keeps the walk's order of additions, and so its bits.)  In place, to
+// the entries with the lower photon first; `rows`: R2 too (n = 4).
+template <class R, int N, int WARPS>
+__device__ __forceinline__ void warp_add_orders(const WarpTables<R, N, WARPS>& tb, int l, bool rows) {
+    constexpr int LP = WarpTables<R, N, WARPS>::LP, NU = N * (N - 1) / 2;
+    for (int it = l; it < (rows ? 8 : 4) * NU; it += LP) {
+        Row<R>* t = it < 4 * NU ? tb.PC : tb.R2;
+        const int q = it < 4 * NU ? it : it - 4 * NU;
+        int x, y;
+        pair_of_unit<N>(q >> 2, x, y);
+        Row<R>* d = t + 4 * pair_slot<N>(x, y) + (q & 3);
+        const Row<R> a = ld_row(d), b = ld_row(t + 4 * pair_slot<N>(y, x) + (q & 3));
+        st_row(d, Row<R>{a.ar + b.ar, a.ai + b.ai, a.br + b.br, a.bi + b.bi});
+    }
+}
+
 // The same contract as amplitude_rounds_lanes; BLOCK threads, whole warps.
 // With BAR = 0 the block meets once at the end; the consumers of a
 // warp-specialised block (BAR != 0) meet their producers right after, and the
@@ -223,6 +244,7 @@ __device__ __forceinline__ void amplitude_rounds_warps(unsigned char* table_smem
     using WT = WarpTables<R, N, BLOCK / 32>;
     constexpr int NS = WT::NS, PB = WT::PB, PW = WT::PW, LP = WT::LP, NW = BLOCK / 32;
     constexpr unsigned FULL = NS - 1;
+    constexpr bool kAdd = sizeof(R) != sizeof(float);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char* mem = table_smem + (size_t)warp * (WT::bytes / NW);
     const WT tb(mem, lane / LP);
@@ -250,6 +272,11 @@ __device__ __forceinline__ void amplitude_rounds_warps(unsigned char* table_smem
         __syncwarp();
         if (mine) warp_pairs(tb, l);
         __syncwarp();
+        if constexpr (kAdd) {
+            // (at n = 5 the rows after two photons are extended one by one, so only the columns are added)
+            if (mine) warp_add_orders(tb, l, N == 4);
+            __syncwarp();
+        }
         if constexpr (N == 4) {
             // (rolled over the point groups: written out side by side for more
             // independent chains it ran 4 % slower, and so did the table phases
@@ -262,12 +289,13 @@ __device__ __forceinline__ void amplitude_rounds_warps(unsigned char* table_smem
 #pragma unroll
                 for (int k = 0; k < WT::NP; ++k) {
                     const int j1 = k / (N - 1), t = k - j1 * (N - 1), j2 = t + (t >= j1);
+                    if (kAdd && j1 > j2) continue;
                     const unsigned rem = FULL & ~((1u << j1) | (1u << j2));
                     const int a = __ffs(rem) - 1, b = __ffs(rem & (rem - 1)) - 1;
                     const int o = j1 < j2 ? o2(j1, j2) : o2(j2, j1);
                     const Row<R> r = ld_row(tc.R2 + 4 * k + o);
                     close_row(r, ld_row(tc.PC + 4 * pair_slot<N>(a, b) + o2(a, b)), ar, ai);
-                    close_row(r, ld_row(tc.PC + 4 * pair_slot<N>(b, a) + o2(a, b)), ar, ai);
+                    if (!kAdd) close_row(r, ld_row(tc.PC + 4 * pair_slot<N>(b, a) + o2(a, b)), ar, ai);
                 }
                 finish(ar, ai, base + s * PW + lane / NS);
             }
@@ -305,7 +333,7 @@ __device__ __forceinline__ void amplitude_rounds_warps(unsigned char* table_smem
                         const int lo = x < y ? x : y, hi = x < y ? y : x;
                         const Row<R> r = ld_row(r3 + 8 * q + ((ho >> lo & 1u) << 1 | (ho >> hi & 1u) << 2));
                         close_row(r, ld_row(tc.PC + po[u][0]), are[s], aim[s]);
-                        close_row(r, ld_row(tc.PC + po[u][1]), are[s], aim[s]);
+                        if (!kAdd) close_row(r, ld_row(tc.PC + po[u][1]), are[s], aim[s]);
                     }
                 }
                 __syncwarp();
