@@ -211,7 +211,7 @@ __device__ __forceinline__ void input_to_rec(const double* __restrict__ row, con
     double sp = 1;
     for (int a = 2; a < N; ++a) sp *= is;
     rec.fac = ph.cpl * sp;
-    rec.wfac = 0;
+    rec.wfac = is;   // (no event weight here: row_view reads it)
     rec.valid = ok;
     rec.mask = 1;
     rec.tries = 1;
@@ -250,14 +250,15 @@ __device__ __forceinline__ void denominators_parallel(PointRec<R, N>* recs, int 
 }
 
 // Staged input row c (stride srow) as a view for denominators_parallel: the
-// photons, the energies of p1 and p2 and 1/s-hat as input_to_rec forms them (a row it
-// refuses is never evaluated).
-__device__ __forceinline__ MomView row_view(double* stage, int srow, int c, double& E1, double& E2, double& is) {
+// photons, the energies of p1 and p2 and 1/s-hat as input_to_rec leaves it in
+// the record (a row it refuses is never evaluated).
+template <class R, int N>
+__device__ __forceinline__ MomView row_view(double* stage, int srow, const PointRec<R, N>* recs, int c, double& E1,
+                                            double& E2, double& is) {
     double* row = stage + (size_t)c * srow;
     E1 = row[0];
     E2 = row[4];
-    const double s = 2.0 * (row[0] * row[4] - row[3] * row[7]);
-    is = s > 0 ? 1.0 / s : 1.0;
+    is = recs[c].wfac;
     return MomView{row + 8, 1, 4};
 }
 
@@ -295,8 +296,9 @@ amp2_kernel(const double* __restrict__ mom, long long npts, const uint32_t* __re
         __syncthreads();
         for (int t = threadIdx.x; t < cnt; t += BLOCK) input_to_rec<R, N>(stage + t * SROW, ph, recs[t], flag);
         if constexpr (N >= 6) {
+            __syncthreads();
             denominators_parallel<R, N, true, false>(recs, cnt, threadIdx.x, BLOCK, [&](int c, double& E1, double& E2, double& is) {
-                return row_view(stage, SROW, c, E1, E2, is);
+                return row_view(stage, SROW, recs, c, E1, E2, is);
             });
         }
         __syncthreads();
@@ -332,8 +334,9 @@ ward_kernel(const double* __restrict__ mom, long long npts, int ward, double* __
         __syncthreads();
         for (int t = threadIdx.x; t < cnt; t += BLOCK) input_to_rec<R, N>(stage + t * SROW, ph, recs[t], flag);
         if constexpr (N >= 6) {
+            __syncthreads();
             denominators_parallel<R, N, true, false>(recs, cnt, threadIdx.x, BLOCK, [&](int c, double& E1, double& E2, double& is) {
-                return row_view(stage, SROW, c, E1, E2, is);
+                return row_view(stage, SROW, recs, c, E1, E2, is);
             });
         }
         __syncthreads();
@@ -579,8 +582,9 @@ amp2_list_kernel(const double* __restrict__ mom, const int* __restrict__ list, c
         __syncthreads();
         for (int t = threadIdx.x; t < cnt; t += BLOCK) input_to_rec<double, N>(stage + t * SROW, ph, recs[t], flag);
         if constexpr (N >= 6) {
+            __syncthreads();
             denominators_parallel<double, N, true, false>(recs, cnt, threadIdx.x, BLOCK, [&](int c, double& E1, double& E2, double& is) {
-                return row_view(stage, SROW, c, E1, E2, is);
+                return row_view(stage, SROW, recs, c, E1, E2, is);
             });
         }
         __syncthreads();

@@ -79,22 +79,37 @@ __host__ __device__ constexpr int meet_in_offset(int n, int k) {
     return o;
 }
 
-// Group shape: threads per group (two to four warps from n = 6, the whole
-// block below), points a group takes per round, sets T of size m per chunk.
+// Group shape: threads per group, points a group takes per round, sets T of
+// size m per chunk.  FP32: two to four warps from n = 6 (the whole block below)
+// with one point a round.  FP64 from n = 6 is bound by its pipe, so its items
+// fill whole warps: at n = 6 four points of a 128-thread group (160 J and 160 R
+// items of the chunk: five warps each; 80 of 96 lanes with two points of 64
+// threads), at n = 7, 8 two points of the whole block, and at n = 8 12 sets a
+// chunk (three a contraction group; 14 leave two of 16 idle).  GB300, before ->
+// after, heget_amp2 in FP64: 20,001 rows at n = 6 1886 -> 1456 us, 20,011 at n = 7
+// 4617 -> 4017, 5001 at n = 8 4007 -> 3780, of which about a third from these
+// shapes, the rest from the shared set sums, the series reciprocals and the
+// one-photon currents in a phase of their own (each was formed by one lane from
+// the record, two set rows and a photon row, while the other warps waited;
+// FP32, same bits: 50,001 rows at n = 6 348 -> 302 us, 20,001 at n = 7 335 -> 307,
+// at n = 8 741 -> 706).
 template <class R>
 __host__ __device__ constexpr int meet_group_threads(int n, int block) {
-    const int want = n <= 5 ? block : n == 6 ? 64 : 128;
+    const bool f64 = sizeof(R) != sizeof(float);
+    const int want = n <= 5 ? block : n == 6 ? (f64 ? 128 : 64) : f64 ? 256 : 128;
     return want < block ? want : block;
 }
-// (FP64 at n = 6: two points per group, whose longer FP64 phases then
-// share each barrier; in FP32 one point per group is faster.)
 template <class R>
 __host__ __device__ constexpr int meet_group_points(int n, int gth) {
-    const int p = n <= 5 ? gth / 16 : n == 6 && sizeof(R) != sizeof(float) ? 2 : 1;
-    const int q = n <= 5 && sizeof(R) != sizeof(float) ? p / 2 : p;
+    const bool f64 = sizeof(R) != sizeof(float);
+    const int p = n <= 5 ? gth / 16 : !f64 ? 1 : n == 6 ? gth / 32 : gth / 128;
+    const int q = n <= 5 && f64 ? p / 2 : p;
     return q > 0 ? q : 1;
 }
-__host__ __device__ constexpr int meet_chunk(int n) { return n == 8 ? 14 : set_binom(n, n / 2); }
+template <class R>
+__host__ __device__ constexpr int meet_chunk(int n) {
+    return n == 8 ? (sizeof(R) == sizeof(float) ? 14 : 12) : set_binom(n, n / 2);
+}
 
 template <class R, int N, int BLOCK>
 struct MeetTables {
@@ -105,7 +120,7 @@ struct MeetTables {
     static constexpr int G = BLOCK / GTH;
     static constexpr int PG = meet_group_points<R>(N, GTH);
     static constexpr int CM = set_binom(N, M), CMK = set_binom(N, MK);
-    static constexpr int CH = meet_chunk(N);
+    static constexpr int CH = meet_chunk<R>(N);
     // rows per point: two buffers per side, alternating by size: J of size
     // M-2 (M-4, ...) and then the chunk's J of size M in the first, M-1
     // (M-3, ...) in the second; K of size MK-1 (MK-3, ...), MK-2 (...); the
@@ -122,11 +137,12 @@ struct MeetTables {
     static constexpr int GT = GTH / (PG * CT) > 0 ? GTH / (PG * CT) : 1;
     static constexpr int HM = 1 << (N - CB);             // values of the helicity bits above CB
     static constexpr int NIN = meet_in_offset(N, MK + 1);
-    // the groups' amplitudes overlay J1, K0, K1 of the group's point once the
-    // last chunk's currents are formed (one point per group), else follow
-    static constexpr size_t XAB = (size_t)GT * PG * NS * 2 * sizeof(R);
-    static constexpr bool XA_OVER = PG == 1 && XAB <= (size_t)(J1 + K0 + K1) * sizeof(Row<R>);
-    static constexpr size_t GB = (size_t)PG * PT * sizeof(Row<R>) + (XA_OVER ? 0 : XAB);   // bytes per group
+    // the contraction groups' amplitudes of a point overlay its J1, K0, K1 once
+    // the last chunk's currents are formed, or follow where those are too small
+    static constexpr size_t XAP = (size_t)GT * NS * 2;   // per point, of R
+    static constexpr size_t XAB = XAP * sizeof(R);
+    static constexpr bool XA_OVER = XAB <= (size_t)(J1 + K0 + K1) * sizeof(Row<R>);
+    static constexpr size_t GB = (size_t)PG * PT * sizeof(Row<R>) + (XA_OVER ? 0 : PG * XAB);   // bytes per group
     static_assert(N >= 2 && PG * CT * GT <= GTH, "group shape");
     static constexpr size_t align4(size_t x) { return (x + 3) & ~(size_t)3; }
     static constexpr size_t bytes = (size_t)G * GB + align4((size_t)NIN * 2) + 2 * (size_t)NS + (size_t)HM * HM + 80;
@@ -156,9 +172,9 @@ struct MeetTables {
         return LV(g, p) + J0 + J1 + (((MK - 1 - k) & 1) ? K0 : 0);
     }
     __device__ __forceinline__ Row<R>* RV(int g, int p) const { return LV(g, p) + J0 + J1 + K0 + K1; }
-    __device__ __forceinline__ R* XA(int g) const {
-        return XA_OVER ? reinterpret_cast<R*>(LV(g, 0) + J0)
-                       : reinterpret_cast<R*>(base + (size_t)g * GB + (size_t)PG * PT * sizeof(Row<R>));
+    __device__ __forceinline__ R* XA(int g, int p) const {
+        return XA_OVER ? reinterpret_cast<R*>(LV(g, p) + J0)
+                       : reinterpret_cast<R*>(base + (size_t)g * GB + (size_t)PG * PT * sizeof(Row<R>)) + p * XAP;
     }
 };
 
@@ -453,6 +469,57 @@ __device__ __forceinline__ void meet_contract(int TL, const Row<R>* J, const Row
 #undef HEGET_MEET_CASE
 }
 
+// Photon directions and set data of a group's points, by its threads.  FP64
+// from n = 6 takes four sets an item (the sets that differ in photons 0 and 1
+// share the sum over the others: 8 additions a set instead of 4 n).
+template <class R, int N, int BLOCK>
+__device__ __forceinline__ void meet_photons_and_sets(const MeetTables<R, N, BLOCK>& tb, int g, int lid,
+                                                      const PointRec<R, N>* rb, int cnt) {
+    using MT = MeetTables<R, N, BLOCK>;
+    constexpr int PG = MT::PG, NS = MT::NS;
+    constexpr bool kQuads = sizeof(R) != sizeof(float) && N >= 6;
+    constexpr int NI = N + (kQuads ? NS / 4 : NS);
+    constexpr unsigned FULL = NS - 1;
+    for (int it = lid; it < PG * NI; it += MT::GTH) {
+        const int p = it / NI, e = it - p * NI;
+        if (p >= cnt) continue;
+        const PointRec<R, N>& rc = rb[p];
+        if (e < N) {
+            st_row(tb.PH(g, p) + e, photon_row<R>(rc.k[e]));
+        } else if constexpr (!kQuads) {
+            const unsigned T = tb.LIST[e - N];
+            if (T != 0u && T != FULL) st_row(tb.SD(g, p) + T, set_row<R, N>(rc, T));
+        } else {
+            const unsigned T0 = 4u * (unsigned)(e - N);
+            R q0 = -rc.e2, q1 = R(0), q2 = R(0), q3 = rc.e2;
+#pragma unroll
+            for (int i = 2; i < N; ++i)
+                if (T0 >> i & 1) {
+                    q0 += rc.k[i][0];
+                    q1 += rc.k[i][1];
+                    q2 += rc.k[i][2];
+                    q3 += rc.k[i][3];
+                }
+            // photons 0 and 1 in Gray-code order: none, 0, 0 and 1, 1
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                if (m > 0) {
+                    const R* k = rc.k[m == 2 ? 1 : 0];
+                    const R s = m == 3 ? R(-1) : R(1);
+                    q0 = fmad<R>(s, k[0], q0);
+                    q1 = fmad<R>(s, k[1], q1);
+                    q2 = fmad<R>(s, k[2], q2);
+                    q3 = fmad<R>(s, k[3], q3);
+                }
+                const unsigned T = T0 | (m ^ (m >> 1));
+                if (T == 0u || T == FULL) continue;
+                const R it_ = recip<R>(rc.t[T]);
+                st_row(tb.SD(g, p) + T, Row<R>{(q0 + q3) * it_, (q0 - q3) * it_, q1 * it_, q2 * it_});
+            }
+        }
+    }
+}
+
 // Amplitude rounds over recs[0 .. cnt-1] by the met-in-the-middle recursion:
 // the same contract as amplitude_rounds (recs[p].ssum = sum_h w_h |A_h|^2 in
 // the scaled units of the records; mask: helicity mask, NULL = all).  All
@@ -475,32 +542,27 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
         for (int base = g * PG; base < cnt; base += G * PG) {
             const int rc = min(PG, cnt - base);
             const PointRec<R, N>* rb = recs + base;
-            // photon and set data; E and the one-photon currents (helicity-major,
-            // row lambda N + i): J({i}) = n2 (e10, -e00) Q_{i}, E u_R = n1 (e00, e10),
-            // K({i}) = Q_{all - i} E u_R (or R = E u_R at n = 2), from the record
-            for (int it = lid; it < PG * (N + NS + 2 * N); it += GTH) {
-                const int p = it / (N + NS + 2 * N), e = it - p * (N + NS + 2 * N);
-                if (p >= rc) continue;
-                const PointRec<R, N>& rc_ = rb[p];
-                if (e < N) {
-                    tb.PH(g, p)[e] = photon_row<R>(rc_.k[e]);
-                } else if (e < N + NS) {
-                    const unsigned T = tb.LIST[e - N];
-                    if (T != 0u && T != FULL) tb.SD(g, p)[T] = set_row<R, N>(rc_, T);
-                } else if (rc_.valid) {
-                    const int q = e - N - NS, lam = q & 1, i = q >> 1;
-                    const EMat<R> E = e_matrix<R>(photon_row<R>(rc_.k[i]), lam);
-                    Row<R>* em = tb.E(g, p) + 2 * lam * N + i;
-                    st_row(em, Row<R>{E.e00, E.e01r, E.e01i, E.e10r});
-                    st_row(em + N, Row<R>{E.e10i, R(0), R(0), R(0)});
-                    const R n1 = rc_.n1, n2 = rc_.n2;
-                    const int x = lam * N + i;
-                    st_row(tb.J(g, p, 1) + x,
-                           row_q<R>(Row<R>{n2 * E.e10r, n2 * E.e10i, -n2 * E.e00, R(0)}, set_row<R, N>(rc_, 1u << i)));
-                    const Row<R> cl{n1 * E.e00, R(0), n1 * E.e10r, n1 * E.e10i};
-                    if constexpr (MK >= 2) st_row(tb.K(g, p, 1) + x, q_col<R>(set_row<R, N>(rc_, FULL & ~(1u << i)), cl));
-                    else st_row(tb.RV(g, p) + lam * N + (N - 1 - i), cl);   // n = 2: at the place of T = all - {i}
-                }
+            // photon and set data
+            meet_photons_and_sets(tb, g, lid, rb, rc);
+            meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);
+            // E and the one-photon currents (helicity-major, row lambda N + i):
+            // J({i}) = n2 (e10, -e00) Q_{i}, E u_R = n1 (e00, e10), K({i}) = Q_{all - i} E u_R
+            // (or R = E u_R at n = 2)
+            for (int it = lid; it < PG * 2 * N; it += GTH) {
+                const int p = it / (2 * N), q = it - p * 2 * N;
+                if (p >= rc || !rb[p].valid) continue;
+                const int lam = q & 1, i = q >> 1;
+                const EMat<R> E = e_matrix<R>(ld_row(tb.PH(g, p) + i), lam);
+                Row<R>* em = tb.E(g, p) + 2 * lam * N + i;
+                st_row(em, Row<R>{E.e00, E.e01r, E.e01i, E.e10r});
+                st_row(em + N, Row<R>{E.e10i, R(0), R(0), R(0)});
+                const R n1 = rb[p].n1, n2 = rb[p].n2;
+                const int x = lam * N + i;
+                st_row(tb.J(g, p, 1) + x, row_q<R>(Row<R>{n2 * E.e10r, n2 * E.e10i, -n2 * E.e00, R(0)},
+                                                   ld_row(tb.SD(g, p) + (1u << i))));
+                const Row<R> cl{n1 * E.e00, R(0), n1 * E.e10r, n1 * E.e10i};
+                if constexpr (MK >= 2) st_row(tb.K(g, p, 1) + x, q_col<R>(ld_row(tb.SD(g, p) + (FULL & ~(1u << i))), cl));
+                else st_row(tb.RV(g, p) + lam * N + (N - 1 - i), cl);   // n = 2: at the place of T = all - {i}
             }
             meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);
             if constexpr (MK >= 3) meet_phase<R, N, BLOCK, BAR, GBAR0, 2>(tb, g, lid, rb, rc);
@@ -532,11 +594,11 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
                 }
                 if (c0 + CH < CM) meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);   // before the next chunk's currents
             }
-            // the groups' amplitudes, configuration-major (entry ((u PG + p) 2^CB
-            // + b) CT + hi for lambda = (hi << CB) | b): a warp's lanes store
+            // the groups' amplitudes, configuration-major (entry (u 2^CB + b) CT + hi
+            // of the point for lambda = (hi << CB) | b): a warp's lanes store
             // consecutive words
             if (mine) {
-                R* xa = tb.XA(g) + (((size_t)gt * PG + p) << CB) * CT * 2 + (size_t)hi * 2;
+                R* xa = tb.XA(g, p) + ((size_t)gt << CB) * CT * 2 + (size_t)hi * 2;
 #pragma unroll
                 for (int b = 0; b < (1 << CB); ++b) {
                     using V2 = typename std::conditional<sizeof(R) == sizeof(float), float2, double2>::type;
@@ -561,7 +623,7 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
                         R ar = R(0), ai = R(0);
 #pragma unroll
                         for (int u = 0; u < GT; ++u) {
-                            const R* a = tb.XA(g) + ((((size_t)u * PG + q) << CB) + b) * CT * 2 + (size_t)hh * 2;
+                            const R* a = tb.XA(g, q) + (((size_t)u << CB) + b) * CT * 2 + (size_t)hh * 2;
                             ar += a[0];
                             ai += a[1];
                         }
