@@ -298,6 +298,12 @@ int subset_amp2_tile(int n, int precision) {
     return precision == HEGET_FP64 ? t64[n] : t32[n];
 }
 
+// Points per tile of the fused tile kernel: the tree's, and for the FP64
+// subset recursion at n = 8 as many as keep its groups of records full.
+int xsec_default_tile(int n, int precision, int alg) {
+    return alg == kAlgSubset && precision == HEGET_FP64 && n == 8 ? 32 : default_tile(n, true);
+}
+
 int xsec_shape_count(int n, int precision, int alg) {
     return precision == HEGET_FP32 && alg == kAlgTree && n >= 6 ? 4 : 1;
 }
@@ -328,7 +334,9 @@ int default_amp_launch(int n, int precision, long long npts, int num_sms, AmpLau
     L->block = xsec && precision == HEGET_FP32 && alg != kAlgSubset && (n == 6 || n == 7) ? (n == 6 ? 160 : 224)
                                                                                         : kBlockThreads;
     if (L->shape > 0) L->block = tree_tile_shape(n, L->shape).block;
-    L->tile = tile > 0 ? tile : !xsec && alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, xsec);
+    L->tile = tile > 0 ? tile
+            : xsec     ? xsec_default_tile(n, precision, alg)
+            : alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, false);
     const bool sub = alg == kAlgSubset;
     const int e = precision == HEGET_FP32
                       ? (sub ? occupancy_alg<float, kAlgSubset>(n, L->tile, &bpsm, &smem)
@@ -481,7 +489,8 @@ int batch_default_tile(int n, int precision, int alg) {
     // subset recursion: the largest tile whose block (records, staging and
     // the recursion's tables) still lets two blocks share an SM, up to 128
     static const int sub32[9] = {0, 0, 128, 128, 128, 64, 64, 64, 64};
-    static const int sub64[9] = {0, 0, 128, 128, 64, 16, 8, 8, 8};
+    // (FP64 from n = 6: rec_chunk records of a larger tile at a time)
+    static const int sub64[9] = {0, 0, 128, 128, 64, 16, 64, 32, 32};
     if (alg != kAlgSubset) return default_tile(n, true);
     return precision == HEGET_FP64 ? sub64[n] : sub32[n];
 }
@@ -685,7 +694,8 @@ int heget_get_tile(const heget_ctx* ctx, int n, int precision, int kind) {
     if (!ctx || n < kMinN || n > kMaxN || (kind != 0 && kind != 1)) return -1;
     const int t = ctx->tiles[kind][precision == HEGET_FP64][n];
     if (t > 0) return t;
-    return kind == 0 && ctx->alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, kind == 1);
+    if (kind == 1) return xsec_default_tile(n, precision, ctx->alg);
+    return ctx->alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, false);
 }
 
 int heget_set_params(heget_ctx* ctx, const heget_params* p) {
@@ -1068,7 +1078,12 @@ extern "C" int heget_xsec_batch(heget_ctx* ctx, const heget_xsec_request* reqs, 
         std::vector<BatchReq> br;
         std::vector<WorkItem> items;
         size_t smem = 0;
-        for (int i = 0; i < count; ++i) {
+        // requests of many photons first: their tiles run longest, and the last
+        // ones of a launch should be short
+        std::vector<int> order(count);
+        for (int i = 0; i < count; ++i) order[i] = i;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return reqs[a].n > reqs[b].n; });
+        for (int i : order) {
             const heget_xsec_request& q = reqs[i];
             if (q.precision != prec) continue;
             const int tile_o = ctx->tiles[1][prec == HEGET_FP64][q.n];

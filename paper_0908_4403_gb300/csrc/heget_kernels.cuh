@@ -145,6 +145,32 @@ __host__ __device__ constexpr size_t xsec_region_bytes(int tile) {
     constexpr size_t tb = table_bytes<R, N, BLOCK, ALG, HB, G>();
     return tb > st ? tb : st;
 }
+// Records that a fused tile holds at a time: all of its points (0), or, for
+// the FP64 subset recursion from n = 6, whose records are 0.8 to 2.4 KB, fewer
+// than the tile generates.  A quarter to a third of the points pass the cuts,
+// and a round takes 8 points at n = 6 and 2 above: with one tile of 8 points
+// per round most of a block's groups waited.  The generated momenta then keep
+// a place of their own beside the round tables.
+template <class R, int N, int ALG>
+__host__ __device__ constexpr int rec_chunk() {
+    return sizeof(R) == sizeof(double) && ALG == kAlgSubset ? (N == 6 ? 32 : N == 7 ? 24 : N == 8 ? 16 : 0) : 0;
+}
+struct PassedPoint {   // a point that passed the cuts, until its record is built
+    double iM, rs;
+    int idx, hsel;
+};
+template <class R, int N, int BLOCK, int ALG, int HB = -1, int G = -1>
+__host__ __device__ constexpr size_t tile_stage_offset() {
+    return rec_chunk<R, N, ALG>() ? table_bytes<R, N, BLOCK, ALG, HB, G>() : 0;
+}
+template <class R, int N, int BLOCK, int ALG, int HB = -1, int G = -1>
+__host__ __device__ constexpr size_t tile_recs_offset(int tile) {
+    return rec_chunk<R, N, ALG>() ? table_bytes<R, N, BLOCK, ALG, HB, G>() +
+                                        align16((size_t)tile * N * kMomSlots * sizeof(double)) +
+                                        align16((size_t)tile * sizeof(PassedPoint))
+                                  : xsec_region_bytes<R, N, BLOCK, ALG, HB, G>(tile);
+}
+
 template <class R, int N, int BLOCK, int ALG = kAlgAny>
 __host__ __device__ constexpr size_t amp2_smem_bytes(int tile) {
     return amp2_region_bytes<R, N, BLOCK, ALG>(tile) + align16((size_t)tile * sizeof(PointRec<R, N>));
@@ -158,8 +184,15 @@ __host__ __device__ constexpr bool xsec_parks_sums() {
 }
 template <class R, int N, int BLOCK, int ALG = kAlgAny, int HB = -1, int G = -1>
 __host__ __device__ constexpr size_t xsec_smem_bytes(int tile) {
-    return xsec_region_bytes<R, N, BLOCK, ALG, HB, G>(tile) + align16((size_t)tile * sizeof(PointRec<R, N>)) +
+    constexpr int chunk = rec_chunk<R, N, ALG>();
+    return tile_recs_offset<R, N, BLOCK, ALG, HB, G>(tile) +
+           align16((size_t)(chunk ? chunk : tile) * sizeof(PointRec<R, N>)) +
            (xsec_parks_sums<R, N>() ? (size_t)BLOCK * sizeof(Partial) : 0);
+}
+// The FP64 recomputation of escalated points: every record of its tile.
+template <int N, int BLOCK>
+__host__ __device__ constexpr size_t escalate_smem_bytes(int tile) {
+    return xsec_region_bytes<double, N, BLOCK, kAlgSubset>(tile) + align16((size_t)tile * sizeof(PointRec<double, N>));
 }
 
 // FP32 -> FP64 escalation lists of a fused launch: block b appends the
@@ -382,10 +415,12 @@ __device__ __forceinline__ void xsec_tile(unsigned char* smem, int tile, uint64_
                                           const SamplerArgs& S, const Physics& ph, Partial& acc,
                                           double* __restrict__ w_out, const EscArgs& esc, int& esc_n) {
     __shared__ int s_cnt[BLOCK / 32];
-    double* stage = reinterpret_cast<double*>(smem);
     constexpr bool kEsc = ESC && sizeof(R) == sizeof(float);
-    PointRec<R, N>* recs =
-        reinterpret_cast<PointRec<R, N>*>(smem + xsec_region_bytes<R, N, BLOCK, table_alg<ALG, kEsc>(), HB, G>(tile));
+    constexpr int TAB = table_alg<ALG, kEsc>(), kChunk = rec_chunk<R, N, TAB>();
+    double* stage = reinterpret_cast<double*>(smem + tile_stage_offset<R, N, BLOCK, TAB, HB, G>());
+    PointRec<R, N>* recs = reinterpret_cast<PointRec<R, N>*>(smem + tile_recs_offset<R, N, BLOCK, TAB, HB, G>(tile));
+    [[maybe_unused]] PassedPoint* passed = reinterpret_cast<PassedPoint*>(
+        reinterpret_cast<unsigned char*>(recs) - align16((size_t)tile * sizeof(PassedPoint)));   // (with kChunk)
     int npass = 0;
     for (int t0 = 0; t0 < cnt; t0 += BLOCK) {
         const int t = t0 + (int)threadIdx.x;
@@ -403,14 +438,46 @@ __device__ __forceinline__ void xsec_tile(unsigned char* smem, int tile, uint64_
         int tot;
         const int pos = compact_pos<BLOCK>(pass, threadIdx.x, s_cnt, 0, tot);
         if (pass) {
-            recs[npass + pos].idx = t;
-            recs[npass + pos].hsel = point_hsel<N>(ph, seed, (uint64_t)(first + t));
-            recs[npass + pos].fac = ev.iM;   // 1/M and sqrt(s-hat) until the record is built
-            recs[npass + pos].wfac = ev.rs;
+            const int hsel = point_hsel<N>(ph, seed, (uint64_t)(first + t));
+            if constexpr (kChunk > 0) {
+                passed[npass + pos] = PassedPoint{ev.iM, ev.rs, t, hsel};
+            } else {
+                recs[npass + pos].idx = t;
+                recs[npass + pos].hsel = hsel;
+                recs[npass + pos].fac = ev.iM;   // 1/M and sqrt(s-hat) until the record is built
+                recs[npass + pos].wfac = ev.rs;
+            }
         }
         npass += tot;
     }
     __syncthreads();
+    if constexpr (kChunk > 0) {
+        for (int c0 = 0; c0 < npass; c0 += kChunk) {
+            const int nc = min(kChunk, npass - c0);
+            for (int c = threadIdx.x; c < nc; c += BLOCK) {
+                const PassedPoint q = passed[c0 + c];
+                recs[c].idx = q.idx;
+                recs[c].hsel = q.hsel;
+                pass_to_rec<R, N>(MomView{stage + q.idx, tile, kMomSlots}, q.iM, q.rs, ph, recs[c]);
+            }
+            __syncthreads();
+            denominators_parallel<R, N, false, true>(recs, nc, threadIdx.x, BLOCK, [&](int c, double& E1, double& E2, double& is) {
+                E1 = E2 = 0.5;
+                is = 1.0;
+                return MomView{stage + recs[c].idx, tile, kMomSlots};
+            });
+            __syncthreads();
+            amp_rounds<R, N, BLOCK, 0, ALG, HB, G>(smem, recs, nc, nullptr, ph.alg);   // ends with a block barrier
+            for (int c = threadIdx.x; c < nc; c += BLOCK) {
+                const double w = (double)recs[c].ssum * recs[c].wfac;
+                acc.sw = dd_add_d(acc.sw, w);
+                acc.sw2 = dd_add_d(acc.sw2, w * w);
+                if (w_out) w_out[recs[c].idx] = w;
+            }
+        }
+        __syncthreads();   // the momenta are read: the next tile may generate
+        return;
+    }
     // records built one per thread in compacted order: every lane busy
     for (int c = threadIdx.x; c < npass; c += BLOCK) {
         PointRec<R, N>& rec = recs[c];

@@ -163,7 +163,7 @@ template <int N>
 static int launch_escalate_n(uint64_t seed, long long i0, const SamplerArgs& S, const Physics& ph, int tile,
                              const EscArgs& esc, Partial* out, double* w_out, int grid, cudaStream_t st) {
     auto k = xsec_escalate_kernel<N, kBlock>;
-    const size_t smem = xsec_smem_bytes<double, N, kBlock, kAlgSubset>(tile);
+    const size_t smem = escalate_smem_bytes<N, kBlock>(tile);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     k<<<grid, kBlock, smem, st>>>(seed, i0, S, ph, tile, esc, out, w_out);
