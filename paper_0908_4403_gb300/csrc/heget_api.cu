@@ -298,10 +298,18 @@ int subset_amp2_tile(int n, int precision) {
     return precision == HEGET_FP64 ? t64[n] : t32[n];
 }
 
-// Points per tile of the fused tile kernel: the tree's, and for the FP64
-// subset recursion at n = 8 as many as keep its groups of records full.
+// Points per tile of the fused tile kernel.  FP64: tiles that leave room for
+// two blocks an SM (n = 4, 5), and small ones where a tile runs long (n = 8 in
+// records of rec_chunk; GB300 sweep, default -> here: tree n = 4, 262,144 points 1805 ->
+// 1598 us, n = 5, 65,536 points 2306 -> 2129; subset n = 5 1085 -> 938, n = 8, 8192
+// points 1615 with 32 -> 1413).
 int xsec_default_tile(int n, int precision, int alg) {
-    return alg == kAlgSubset && precision == HEGET_FP64 && n == 8 ? 32 : default_tile(n, true);
+    if (precision == HEGET_FP64) {
+        if (n == 4 && alg != kAlgSubset) return 96;
+        if (n == 5) return 32;
+        if (n == 8 && alg == kAlgSubset) return 16;
+    }
+    return default_tile(n, true);
 }
 
 int xsec_shape_count(int n, int precision, int alg) {
@@ -490,7 +498,7 @@ int batch_default_tile(int n, int precision, int alg) {
     // the recursion's tables) still lets two blocks share an SM, up to 128
     static const int sub32[9] = {0, 0, 128, 128, 128, 64, 64, 64, 64};
     // (FP64 from n = 6: rec_chunk records of a larger tile at a time)
-    static const int sub64[9] = {0, 0, 128, 128, 64, 16, 64, 32, 32};
+    static const int sub64[9] = {0, 0, 128, 128, 128, 32, 64, 32, 16};
     if (alg != kAlgSubset) return default_tile(n, true);
     return precision == HEGET_FP64 ? sub64[n] : sub32[n];
 }
@@ -1257,10 +1265,14 @@ extern "C" int heget_xsec_noalloc(int device, int n, uint64_t seed, int64_t i0, 
     // kernel with its default tile, whose grid bounds N
     if ((r = default_amp_launch(n, precision, N > 0 ? N : 1, sms, &L, true, 0)))
         return cuda_fail((cudaError_t)r, "occupancy");
-    if (N > 0 && L.grid > kNoAllocMaxBlocks)
+    // FP64 at n = 4, 5 runs smaller tiles than the range was set for: its blocks
+    // take several tiles each beyond 4096
+    const long long max_points = (long long)kNoAllocMaxBlocks * default_tile(n, true);
+    if (N > 0 && !L.ws && N > max_points)
         return fail(HEGET_EINVAL,
-                    "N = %lld needs %d block partials; the no-allocation path holds %d (N <= %lld at n = %d)",
-                    (long long)N, L.grid, kNoAllocMaxBlocks, (long long)kNoAllocMaxBlocks * L.tile, n);
+                    "N = %lld needs more block partials than the %d of the no-allocation path (N <= %lld at n = %d)",
+                    (long long)N, kNoAllocMaxBlocks, max_points, n);
+    L.grid = std::min(L.grid, kNoAllocMaxBlocks);
     Partial* scratch = nullptr;
     if ((r = noalloc_scratch(device, &scratch))) return r;
     const Physics ph = physics_of(p, n);

@@ -118,6 +118,9 @@ __device__ __forceinline__ void amp_rounds(unsigned char* smem, PointRec<R, N>* 
         if constexpr (tree_warp_rounds<R, N, SH::HB>()) {
             amplitude_rounds_warps<R, N, BLOCK, BAR>(smem, recs, cnt, mask);
             if (BAR != 0 && kappa) group_sync<BAR, BLOCK>();   // the bound reuses the warps' tables
+        } else if constexpr (tree_point_rounds<R, N, SH::HB>()) {
+            amplitude_rounds_points<R, N, BLOCK, BAR>(recs, cnt, mask);
+            if (BAR != 0 && kappa) group_sync<BAR, BLOCK>();
         } else {
             amplitude_rounds<R, N, BLOCK, BAR, SH::HB, SH::G>(smem, recs, cnt, mask);
         }
