@@ -5,8 +5,8 @@
 // exponent among them as a 128-bit fixed-point number, the numbers are added
 // as integers, and the total goes back to a double-double.  The additions are
 // exact, so the result does not depend on their order; what is lost are bits
-// below 2^-115 (a warp) or 2^-(120 - log2 terms) (a whole grid) of the largest
-// term, at or below the 2^-104 of a double-double addition.
+// below 2^-113 (a block) or 2^-(124 - log2 terms) (a whole grid) of the largest
+// term, below the 2^-104 of a double-double addition.
 //
 // Why integers: GB300 issues a warp's FP64 instruction in 64 cycles of its
 // sub-partition whatever the number of active lanes, and a double-double
@@ -111,34 +111,10 @@ __host__ __device__ __forceinline__ DD dd_of_fixed(__int128 v, int em, int top) 
     return dd_of_int(v, em - 1075 - top);
 }
 
-constexpr int kWarpTop = 66;   // 64 terms a warp (hi and lo of 32 lanes), one bit to spare
-
 __device__ __forceinline__ __int128 shfl_down128(__int128 v, int off) {
     const unsigned long long l = __shfl_down_sync(0xffffffffu, (unsigned long long)v, off);
     const unsigned long long h = __shfl_down_sync(0xffffffffu, (unsigned long long)((unsigned __int128)v >> 64), off);
     return (__int128)(((unsigned __int128)h << 64) | l);
-}
-
-__device__ __forceinline__ DD warp_sum_dd(const DD& a) {
-    const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a));
-    __int128 v = fixed_of(a, em, kWarpTop);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += shfl_down128(v, off);
-    return dd_of_fixed(v, em, kWarpTop);
-}
-
-// Sum over the 32 lanes of a warp, valid in lane 0.
-__device__ __forceinline__ Partial warp_reduce_partial(Partial a) {
-    a.sw = warp_sum_dd(a.sw);
-    a.sw2 = warp_sum_dd(a.sw2);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        a.npass += __shfl_down_sync(0xffffffffu, a.npass, off);
-        a.ntotal += __shfl_down_sync(0xffffffffu, a.ntotal, off);
-        a.ntries += __shfl_down_sync(0xffffffffu, a.ntries, off);
-        a.nesc += __shfl_down_sync(0xffffffffu, a.nesc, off);
-    }
-    return a;
 }
 
 __device__ __forceinline__ Partial zero_partial() {
@@ -149,16 +125,54 @@ __device__ __forceinline__ Partial zero_partial() {
     return p;
 }
 
-// Sum of the per-thread partials of a block (each warp, then the warps'
-// sums).  Uses `scratch` (BLOCK/32 Partials of shared memory); result valid
-// in thread 0.  All threads must call it.
+// Sum of the per-thread partials of a block: the largest exponents of all
+// threads, the warps' sums as integers aligned to them, one thread adds those.
+// Uses `scratch` (BLOCK/32 Partials of shared memory, 16-byte aligned); result
+// valid in thread 0.  All threads must call it.
+struct alignas(16) WarpSums {
+    __int128 v[2];
+    long long c[4];
+};
+static_assert(sizeof(WarpSums) == sizeof(Partial), "the scratch holds one per warp");
+
 template <int BLOCK>
 __device__ __forceinline__ Partial block_reduce_partial(Partial a, Partial* scratch) {
-    static_assert(BLOCK % 32 == 0 && BLOCK / 32 <= 32, "whole warps, one warp to add them");
-    a = warp_reduce_partial(a);
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = a;
+    static_assert(BLOCK % 32 == 0 && BLOCK <= 1024, "whole warps");
+    constexpr int NW = BLOCK / 32;
+    constexpr int kTop = 61;   // 2 BLOCK <= 2048 terms of a sum below 2^(53 + kTop)
+    __shared__ int s_em[2][NW];
+    WarpSums* sums = reinterpret_cast<WarpSums*>(scratch);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int em[2] = {(int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a.sw)),
+                 (int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a.sw2))};
+    if (lane == 0) {
+        s_em[0][warp] = em[0];
+        s_em[1][warp] = em[1];
+    }
     __syncthreads();
-    if (threadIdx.x < 32) a = warp_reduce_partial(threadIdx.x < BLOCK / 32 ? scratch[threadIdx.x] : zero_partial());
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        em[0] = max(em[0], s_em[0][w]);
+        em[1] = max(em[1], s_em[1][w]);
+    }
+    WarpSums t{{fixed_of(a.sw, em[0], kTop), fixed_of(a.sw2, em[1], kTop)}, {a.npass, a.ntotal, a.ntries, a.nesc}};
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) t.v[q] += shfl_down128(t.v[q], off);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) t.c[q] += __shfl_down_sync(0xffffffffu, t.c[q], off);
+    }
+    if (lane == 0) sums[warp] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll 1
+        for (int w = 1; w < NW; ++w) {
+            for (int q = 0; q < 2; ++q) t.v[q] += sums[w].v[q];
+            for (int q = 0; q < 4; ++q) t.c[q] += sums[w].c[q];
+        }
+        a = Partial{dd_of_fixed(t.v[0], em[0], kTop), dd_of_fixed(t.v[1], em[1], kTop), t.c[0], t.c[1], t.c[2], t.c[3]};
+    }
     return a;
 }
 
