@@ -41,8 +41,7 @@ struct heget_ctx {
     heget_params params{};
     heget::Partial* partials = nullptr;      // kMaxGrid block partials
     int* flag = nullptr;              // device input-check flag
-    heget_xsec_result* res_dev = nullptr;
-    heget_xsec_result* res_host = nullptr;  // pinned
+    heget_xsec_result* res_host = nullptr;  // pinned; written by the device (heget_xsec)
     int last_parts = 0;               // block partials of the last heget_xsec_launch
     int last_kind = 0;                // its sampler kind
     bool last_ws = false;             // it used the warp-specialised kernel
