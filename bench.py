@@ -37,8 +37,8 @@ METRIC = ("u ubar -> n gamma |M|^2 phase-space points/s (points whose |M|^2 is e
           "n=4 workload; FP32 chain, FP64 phase space + accumulation)")
 WORKLOAD = ("u ubar -> 4 gamma, 1,048,576 points/step/GPU, toy-PDF sqrt(s-hat) = 14 TeV sqrt(x1 x2) > 100 GeV "
             "with x ~ x^-1/2 (1-x)^3, cuts pT>20 GeV |eta|<2.5 dR>0.4, all 64 helicities")
-PATH = ("24 orderings on the prefix tree with the two-ended finish, FP32 chain + FP64 RAMBO/cuts/denominators "
-        "+ double-double sigma accumulation")
+PATH = ("24 orderings on the prefix tree with the two-ended finish, FP32 chain + RAMBO (64-bit integer momenta, "
+        "FP64 boost), cuts (FP32 where it decides, else FP64), FP64 denominators + exact and double-double sums")
 PATH_ORACLE = "FP64 CPU oracle: each of the 24 orderings from scratch with 4x4 Dirac matrices, compensated sums"
 
 
@@ -49,23 +49,23 @@ SMS, SM_GHZ = 152, 2.07
 FP32_PEAK = SMS * 128 * 2 * SM_GHZ / 1e3
 FP64_PEAK = SMS * 2 * 2 * SM_GHZ / 1e3
 # FP64 flops executed per point by the fused n = 4 FP32 step (DFMA x 2 +
-# DADD + DMUL, thread-level predicated-on counts from ncu on 262,144 points
-# of this workload): sqrt(s-hat), RAMBO, cuts, and for the points that pass
-# the cuts the denominators, records, weights and double-double sums.
+# DADD + DMUL, thread-level predicated-on counts from ncu on 1,048,576 points
+# of this workload): sqrt(s-hat), RAMBO's sums and boost, and for the points
+# that pass the cuts the denominators, records, weights and double-double sums.
 # FP64_INSTR_PER_POINT: the same as instructions (DFMA + DADD + DMUL), each
 # taking one slot of the FP64 pipe, 2 per SM and clock.
-FP64_FLOPS_PER_POINT = {4: 671}
-FP64_INSTR_PER_POINT = {4: 516.4}
+FP64_FLOPS_PER_POINT = {4: 177.8}
+FP64_INSTR_PER_POINT = {4: 127.6}
 # DRAM bytes per launch of that kernel (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum): its inputs come from the counter-based generator,
 # so this is code, constant tables and block partials, the same at any size.
-FP64_STEP_TRAFFIC = {4: 152832}
+FP64_STEP_TRAFFIC = {4: 124416}
 
 
 def roofline(n, N, kern_s, peak32_meas, peak64_meas, n_eval=None, subset=False):
-    """Roofline of the fused step's kernel.  At n <= 4 the FP64 pipe binds
-    (the phase space is FP64 by design; one SM retires 2 DFMA per clock
-    against 128 FFMA), above that the FP32 tree does.  n_eval: points whose
+    """Roofline of the fused step's kernel.  At n = 4 the FP64 pipe is its
+    busiest (one SM retires 2 DFMA per clock against 128 FFMA; the boost, the
+    denominators and the sums are FP64), above that the FP32 tree binds.  n_eval: points whose
     amplitudes were evaluated (those that pass the cuts).  subset: the step
     ran the subset recursion (its own flop count, FP32 pipe)."""
     fpp = subset_flops_per_point(n) if subset else tree_flops_per_point(n)
