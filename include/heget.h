@@ -181,15 +181,15 @@ int heget_amp2(heget_ctx* ctx, int n, int64_t N, const double* momenta,
 int heget_ward(heget_ctx* ctx, int n, int64_t N, const double* momenta,
                int photon, int precision, double* ratio, void* stream);
 
-/* The device logarithm of the RAMBO energies q0 = -ln(r r'), Sec. 2.1
- * eq. (4) (Tang's table-driven method, ACM TOMS 16 (1990) 378), exposed so
- * that its accuracy can be checked: y[i] = ln x[i] for N device doubles,
+/* A table-driven FP64 logarithm (Tang, ACM TOMS 16 (1990) 378), once that of
+ * the RAMBO energies q0 = -ln(r r') of Sec. 2.1 eq. (4), which now come from
+ * integer arithmetic of more bits; exposed so that its accuracy can be checked: y[i] = ln x[i] for N device doubles,
  * each a positive normal number (other inputs give unspecified values).
  * Runs on the current device; EINVAL for N < 0 or NULL arrays. */
 int heget_log_table(const double* x, double* y, int64_t N, void* stream);
 
-/* The device cosine and sine of the RAMBO azimuth phi = 2 pi r, Sec. 2.1
- * eq. (4), exposed so that their accuracy can be checked.  words [N][2]
+/* FP64 cosine and sine of an azimuth phi = 2 pi r (once the RAMBO azimuth of
+ * Sec. 2.1 eq. (4)), exposed so that their accuracy can be checked.  words [N][2]
  * (device uint32: lo, hi) are the two random words of one uniform,
  * r = (2m + 1) 2^-53 with m = ((hi << 32) | lo) >> 12 (the generator's layout);
  * cs [N][2] (device doubles) receives (cos phi, sin phi).  Runs on the

@@ -293,7 +293,7 @@ __device__ __forceinline__ void warp_draws(const SamplerArgs& S, uint64_t seed, 
 __device__ __forceinline__ void sample_finish(const SamplerArgs& S, const SampleDraw& d, EventInfo& ev) {
     ev.ok = d.ok();
     ev.tries = d.tries();
-    ev.ua = ev.ub = 1;
+    ev.ua = ev.ub = 1ull << 52;   // e^y = 1, in the middle of FP32's range
     if (S.kind == HEGET_SAMPLER_FIXED) {
         ev.rs = S.sqrt_s;
     } else if (S.kind == HEGET_SAMPLER_UNIFORM) {
@@ -357,7 +357,8 @@ __device__ __forceinline__ R rec_value(double x) {
 // with ln F and ln 2 from double-double tables (heget_logtab.h) and ln(1 + r)
 // by its series to r^6 (|r| <= 2^-9: truncation below 2^-56 relative).  F and
 // e become doubles through their bit patterns, so the whole costs 15 FP64
-// operations instead of a general-purpose logarithm, for the RAMBO energies.
+// operations instead of a general-purpose logarithm.  (An entry point of its
+// own, heget_log_table; the generator's energies come from neg_log.)
 __device__ __forceinline__ double log_table(double x) {
     const int hi = __double2hiint(x), lo = __double2loint(x);
     const int e = ((hi >> 20) & 0x7FF) - 1023;
@@ -388,7 +389,8 @@ __device__ __forceinline__ double log_table(double x) {
 // s = sin theta and c' = cos theta - 1 by their Taylor series (truncated below
 // 1e-19),
 //   cos phi = cos a + (c' cos a - s sin a),  sin phi = sin a + (c' sin a + s cos a),
-// within about 2 ulp; 15 FP64 operations and one table load.
+// within about 2 ulp; 15 FP64 operations and one table load.  (An entry point of
+// its own, heget_sincos_2pi; the generator's azimuth is quadrant_cos_sin.)
 __device__ __forceinline__ void sincos_2pi_words(uint32_t lo, uint32_t hi, double& sp, double& cp) {
     const unsigned long long m = ((((unsigned long long)hi) << 32) | lo) >> 12;
     const unsigned long long j = (m + (1ull << 42)) >> 43;   // 0 .. 512
@@ -450,7 +452,8 @@ __device__ __forceinline__ double rambo(const PointRng& rng, const MomView& v) {
     // M = sqrt(Q^2), b = -Q/M, gamma = Q0/M, a = 1/(1 + gamma) = M/(M + Q0):
     // p_i = (gamma q0 + b.q, q + b (q0 + a b.q)).
     const double M2 = Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3;
-    const double iM = rsqrt_series(M2);
+    // (all photons parallel to rounding: the library's root, NaN below 0)
+    const double iM = __double2hiint(M2) > 0x39B00000 ? rsqrt_series(M2) : rsqrt(M2);   // M2 > 8e-31
     const double M = M2 * iM;
     const double b1 = -Q1 * iM, b2 = -Q2 * iM, b3 = -Q3 * iM;
     const double a = M * recip_series(M + Q0);
@@ -616,15 +619,16 @@ __device__ __forceinline__ float f32_cut(double x) {
 // points at n = 5 668 -> 454 us.
 //
 // The momenta are in RAMBO's units (total M, of the order of n), which FP32
-// holds; pT is compared in GeV.  Energies, pT cuts, e^2E and sinh^2 R that
-// FP32 does not hold are left to pass_cuts, and so is a photon whose pT^2 FP32
+// holds; pT is compared in GeV.  Energies, pT cuts, boosts (u below 2^-30), e^2E
+// and sinh^2 R that FP32 does not hold are left to pass_cuts, and so is a photon whose pT^2 FP32
 // cannot hold accurately.
 template <int N>
 __device__ __forceinline__ int pass_cuts_fast(const MomView& p, const EventInfo& ev, const Physics& ph) {
     constexpr float kU = 5.9604645e-8f;   // 2^-24
     const double scale = ev.rs * ev.iM;
     if (!(ev.rs > 1e-2 && ev.rs < 1e8 && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12 &&
-          !(ph.pt_min > 0 && ph.pt_min < 1e-12)))
+          !(ph.pt_min > 0 && ph.pt_min < 1e-12) &&
+          ev.ua >> 23 != 0 && ev.ub >> 23 != 0))
         return pass_cuts<N>(p, scale, ev.ua, ev.ub, ph);
     constexpr float kLo = 1.0f - 64.0f * kU, kHi = 1.0f + 64.0f * kU;
     // e^y = ua / ub: a and b below are p+ e^y and p- e^-y times ua ub 2^-106
