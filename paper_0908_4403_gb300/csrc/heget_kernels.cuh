@@ -775,22 +775,27 @@ constexpr int kBarDrawFull = 12, kBarDrawEmpty = 14;          // sampler's draws
 // amplitudes, and so does the bound of the escalating kernel, which keeps
 // 256; the subset recursion up to n = 4 and the tree at n = 5 ran 4-16 %
 // slower with 128); 160 for the FP32 tree at n = 6 (five pair-unit slots of two points
-// share out the 15 units evenly); 384 for the subset recursion from n = 7
-// (three groups of four warps, one block per SM).
+// share out the 15 units evenly); 512 for the subset recursion from n = 7
+// (four groups of four warps, one block per SM; 384 with the escalating
+// kernel's error bound, which needs the registers).  GB300, 262144 points,
+// 384 -> 512 consumers with the stages of ws_stage: n = 7 1627 -> 1484 us,
+// n = 8 2767 -> 2654; 65536 points: 506 -> 463, 881 -> 776.
 __host__ __device__ constexpr int ws_consumers(int n, int alg, bool esc) {
-    return n <= 4 && alg == 0 && !esc ? 128 : n == 6 && alg == 0 ? 160 : n >= 7 && alg == 1 ? 384 : 256;
+    return n <= 4 && alg == 0 && !esc ? 128 : n == 6 && alg == 0 ? 160 : n >= 7 && alg == 1 ? (esc ? 384 : 512) : 256;
 }
 // Points per stage (= producer threads, a multiple of 32): as many as the
 // shared memory of the ring, the producers' staging and the round tables
 // allows at two resident blocks per SM; 64 at n = 5, 6, whose FP64
 // generation then spans two warps (one warp leaves the FP64 pipe waiting on
-// its own latencies).  The subset recursion from n = 7 takes 96 with its 384
-// consumers at one block per SM: there the FP64 generation of about four
-// events per evaluated point outweighs the recursion, and three producer
-// warps keep three sub-partitions' FP64 units busy (GB300, n = 8: 8.5e7
-// points/s, from 6.2e7 with 32 producers and two blocks per SM).
+// its own latencies).  The subset recursion from n = 7, at one block per SM,
+// takes 96 at n = 7, where the FP64 generation of about four events per
+// evaluated point outweighs the recursion and three producer warps keep three
+// sub-partitions' FP64 units busy, and 64 at n = 8, where two keep up with
+// the four groups and shared memory holds no more.  GB300, 512 consumers,
+// 262144 points: n = 7 1484 us with 96, 1589 with 64; n = 8 2654 with 64, more
+// with 32.
 __host__ __device__ constexpr int ws_stage(int n, int alg) {
-    return n <= 4 ? 128 : n <= 6 ? 64 : alg == 1 ? 96 : 32;
+    return n <= 4 ? 128 : n <= 6 ? 64 : alg == 1 ? (n == 7 ? 96 : 64) : 32;
 }
 
 // Whether a warp of its own draws for the producers (warp_draws over a whole
