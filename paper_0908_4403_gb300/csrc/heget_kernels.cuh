@@ -770,8 +770,8 @@ constexpr int kBarDrawFull = 12, kBarDrawEmpty = 14;          // sampler's draws
 
 // Consumer threads: 256; 128 for the tree up to n = 4 without the FP32
 // error bound, whose amplitudes are a small share of the block's work (with
-// 256, the consumer warps took issue slots from the FP64 producers: GB300
-// n = 4, 4.98e8 against 4.77e8 evaluated points/s; 96 or 64 starve the
+// 256, the consumer warps take issue slots from the producers: GB300, n = 4,
+// 1,048,576 points 630 us with 128, 771 or more with 192 or 256; 96 or 64 starve the
 // amplitudes, and so does the bound of the escalating kernel, which keeps
 // 256; the subset recursion up to n = 4 and the tree at n = 5 ran 4-16 %
 // slower with 128); 160 for the FP32 tree at n = 6 (five pair-unit slots of two points
