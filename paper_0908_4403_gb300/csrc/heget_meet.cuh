@@ -89,7 +89,7 @@ __host__ __device__ constexpr int meet_in_offset(int n, int k) {
 // after, heget_amp2 in FP64: 20,001 rows at n = 6 1886 -> 1456 us, 20,011 at n = 7
 // 4617 -> 4017, 5001 at n = 8 4007 -> 3780, of which about a third from these
 // shapes, the rest from the shared set sums, the series reciprocals and the
-// one-photon currents in a phase of their own (each was formed by one lane from
+// one-photon currents in a phase of their own from n = 3 (each was formed by one lane from
 // the record, two set rows and a photon row, while the other warps waited;
 // FP32, same bits: 50,001 rows at n = 6 348 -> 302 us, 20,001 at n = 7 335 -> 307,
 // at n = 8 741 -> 706).
@@ -542,9 +542,14 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
         for (int base = g * PG; base < cnt; base += G * PG) {
             const int rc = min(PG, cnt - base);
             const PointRec<R, N>* rb = recs + base;
-            // photon and set data
-            meet_photons_and_sets(tb, g, lid, rb, rc);
-            meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);
+            // photon and set data (n = 2 has no larger sets: its currents come
+            // straight from the records, a phase and a barrier less -- GB300, FP32
+            // heget_amp2 of 12,001 rows 31 us, 35 with the tables; 262,144 rows 128, 140)
+            constexpr bool kDirect = N == 2;
+            if constexpr (!kDirect) {
+                meet_photons_and_sets(tb, g, lid, rb, rc);
+                meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);
+            }
             // E and the one-photon currents (helicity-major, row lambda N + i):
             // J({i}) = n2 (e10, -e00) Q_{i}, E u_R = n1 (e00, e10), K({i}) = Q_{all - i} E u_R
             // (or R = E u_R at n = 2)
@@ -552,14 +557,17 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
                 const int p = it / (2 * N), q = it - p * 2 * N;
                 if (p >= rc || !rb[p].valid) continue;
                 const int lam = q & 1, i = q >> 1;
-                const EMat<R> E = e_matrix<R>(ld_row(tb.PH(g, p) + i), lam);
-                Row<R>* em = tb.E(g, p) + 2 * lam * N + i;
-                st_row(em, Row<R>{E.e00, E.e01r, E.e01i, E.e10r});
-                st_row(em + N, Row<R>{E.e10i, R(0), R(0), R(0)});
+                const EMat<R> E = e_matrix<R>(kDirect ? photon_row<R>(rb[p].k[i]) : ld_row(tb.PH(g, p) + i), lam);
+                if constexpr (!kDirect) {
+                    Row<R>* em = tb.E(g, p) + 2 * lam * N + i;
+                    st_row(em, Row<R>{E.e00, E.e01r, E.e01i, E.e10r});
+                    st_row(em + N, Row<R>{E.e10i, R(0), R(0), R(0)});
+                }
                 const R n1 = rb[p].n1, n2 = rb[p].n2;
                 const int x = lam * N + i;
-                st_row(tb.J(g, p, 1) + x, row_q<R>(Row<R>{n2 * E.e10r, n2 * E.e10i, -n2 * E.e00, R(0)},
-                                                   ld_row(tb.SD(g, p) + (1u << i))));
+                st_row(tb.J(g, p, 1) + x,
+                       row_q<R>(Row<R>{n2 * E.e10r, n2 * E.e10i, -n2 * E.e00, R(0)},
+                                kDirect ? set_row<R, N>(rb[p], 1u << i) : ld_row(tb.SD(g, p) + (1u << i))));
                 const Row<R> cl{n1 * E.e00, R(0), n1 * E.e10r, n1 * E.e10i};
                 if constexpr (MK >= 2) st_row(tb.K(g, p, 1) + x, q_col<R>(ld_row(tb.SD(g, p) + (FULL & ~(1u << i))), cl));
                 else st_row(tb.RV(g, p) + lam * N + (N - 1 - i), cl);   // n = 2: at the place of T = all - {i}
