@@ -338,7 +338,13 @@ amp2_kernel(const double* __restrict__ mom, long long npts, const uint32_t* __re
             });
         }
         __syncthreads();
-        amp_rounds<R, N, BLOCK, 0, ALG>(smem, recs, cnt, mask, ph.alg, esc);
+        bool few = false;
+        if constexpr (ALG == kAlgTree && tree_point_rounds<R, N, ShapeSel<R, N, BLOCK, -1, -1>::HB>()) {
+            static_assert(FewTables<R, N>::bytes <= table_bytes<R, N, BLOCK, ALG>(), "room");
+            few = cnt <= kFewPoints;
+            if (few) amplitude_rounds_few<R, N, BLOCK>(smem, recs, cnt, mask);
+        }
+        if (!few) amp_rounds<R, N, BLOCK, 0, ALG>(smem, recs, cnt, mask, ph.alg, esc);
         const float thr = esc ? esc_threshold(ph.esc_tau) : 0.0f;
         // one thread per point: FP64 normalisation and a coalesced store; points
         // whose FP32 error bound exceeds the threshold are listed for FP64

@@ -47,6 +47,33 @@ __device__ __forceinline__ EHel<R> e_of(const Row<R>& ph, int lam_bit) {
     return EHel<R>{Row<R>{-lam * ph.ar * rs2, -am * ph.br, am * ph.bi, ap * ph.br}, ap * ph.bi};
 }
 
+// The same from a momentum, with 1 -+ lambda cos theta formed from k_z and 1/|k|
+// in one rounding (FP64 at n = 2, 3); every fused operation written out, so
+// that results have the same bits wherever it is inlined.
+template <class R>
+struct PhotonDir {
+    R z, rk, st, cp, sp;   // k_z, 1/|k|, sin theta, cos phi, sin phi
+};
+template <class R>
+__device__ __forceinline__ PhotonDir<R> photon_dir(const R* k) {
+    const R pt2 = fmad<R>(k[1], k[1], k[2] * k[2]), ka2 = fmad<R>(k[3], k[3], pt2);
+    PhotonDir<R> d{k[3], rsq<R>(ka2), R(0), R(1), R(0)};   // (a photon along z: as photon_row)
+    if (pt2 > R(1e-24) * ka2) {
+        const R rpt = rsq<R>(pt2);
+        d.st = pt2 * rpt * d.rk;
+        d.cp = k[1] * rpt;
+        d.sp = k[2] * rpt;
+    }
+    return d;
+}
+template <class R>
+__device__ __forceinline__ EHel<R> e_of(const PhotonDir<R>& d, int lam_bit) {
+    const R rs2 = R(0.70710678118654752440);
+    const R lam = lam_bit ? R(1) : R(-1);
+    const R am = fmad<R>(-lam * d.z, d.rk, R(1)) * rs2, ap = fmad<R>(lam * d.z, d.rk, R(1)) * rs2;
+    return EHel<R>{Row<R>{-lam * d.st * rs2, -am * d.cp, am * d.sp, ap * d.cp}, ap * d.sp};
+}
+
 // step_matrix (of E and a set) and row_times with every fused operation
 // written out: the ones that the compiler makes of the plain forms in the
 // lane-by-lane walk, so that results have the walk's bits whatever the code
@@ -117,6 +144,7 @@ struct WarpTables {
         R3 = PC + 4 * NP;
     }
     __device__ __forceinline__ EHel<R> e(int x) const { return EHel<R>{ld_row(EA + x), EI[x]}; }
+    static __device__ __forceinline__ EHel<R> make_e(const R* k, int lam_bit) { return e_of<R>(photon_row<R>(k), lam_bit); }
 };
 
 // ordered pair k = a (n - 1) + b - [b > a]
@@ -130,19 +158,19 @@ __device__ __forceinline__ void pair_of_slot(int k, int& a, int& b) {
 // Tables of one point by its LP lanes (l), in three phases separated by warp
 // barriers, which the caller places: E and set data; first rows and closures;
 // rows after two photons and pair columns.
-template <class R, int N, int WARPS>
-__device__ __forceinline__ void warp_sets(const WarpTables<R, N, WARPS>& tb, const PointRec<R, N>& rc, int l) {
+template <class R, int N, class WT>
+__device__ __forceinline__ void warp_sets(const WT& tb, const PointRec<R, N>& rc, int l) {
     if (l < 2 * N) {
-        const EHel<R> e = e_of<R>(photon_row<R>(rc.k[l >> 1]), l & 1);
+        const EHel<R> e = WT::make_e(rc.k[l >> 1], l & 1);
         st_row(tb.EA + l, e.a);
         tb.EI[l] = e.e10i;
     }
 #pragma unroll 1
-    for (int T = 1 + l; T < (1 << N) - 1; T += WarpTables<R, N, WARPS>::LP) st_row(tb.SD + T, set_row<R, N>(rc, (unsigned)T));
+    for (int T = 1 + l; T < (1 << N) - 1; T += WT::LP) st_row(tb.SD + T, set_row<R, N>(rc, (unsigned)T));
 }
 
-template <class R, int N, int WARPS>
-__device__ __forceinline__ void warp_ends(const WarpTables<R, N, WARPS>& tb, const PointRec<R, N>& rc, int l) {
+template <class R, int N, class WT>
+__device__ __forceinline__ void warp_ends(const WT& tb, const PointRec<R, N>& rc, int l) {
     if (l < 2 * N) {   // photon l / 2, helicity l % 2
         const EHel<R> e = tb.e(l);
         const Row<R> m1 = step_fused(e, ld_row(tb.SD + (1 << (l >> 1)))).m1;
@@ -152,11 +180,10 @@ __device__ __forceinline__ void warp_ends(const WarpTables<R, N, WARPS>& tb, con
     }
 }
 
-template <class R, int N, int WARPS>
-__device__ __forceinline__ void warp_pairs(const WarpTables<R, N, WARPS>& tb, int l) {
-    constexpr int LP = WarpTables<R, N, WARPS>::LP, NI = 2 * N * (N - 1);
-    constexpr unsigned FULL = (1u << N) - 1;
-    // rows after two photons: items (ordered (j1, j2), helicity of j2)
+// rows after two photons: items (ordered (j1, j2), helicity of j2)
+template <class R, int N, class WT>
+__device__ __forceinline__ void warp_rows(const WT& tb, int l) {
+    constexpr int LP = WT::LP, NI = 2 * N * (N - 1);
 #pragma unroll 1
     for (int it = l; it < NI; it += LP) {
         const int lam = it & 1, k = it >> 1;
@@ -169,6 +196,13 @@ __device__ __forceinline__ void warp_pairs(const WarpTables<R, N, WARPS>& tb, in
         st_row(dst, o0);
         st_row(dst + (x < y ? 1 : 2), o1);
     }
+}
+
+template <class R, int N, int WARPS>
+__device__ __forceinline__ void warp_pairs(const WarpTables<R, N, WARPS>& tb, int l) {
+    constexpr int LP = WarpTables<R, N, WARPS>::LP, NI = 2 * N * (N - 1);
+    constexpr unsigned FULL = (1u << N) - 1;
+    warp_rows<R, N>(tb, l);
     // pair columns: items (ordered (a, b), helicity of a)
 #pragma unroll 1
     for (int it = l; it < NI; it += LP) {
@@ -370,9 +404,9 @@ __device__ __forceinline__ R point_sum(const PointRec<R, N>& rc, const uint32_t*
     EHel<R> e[N][2];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const Row<R> ph = photon_row<R>(rc.k[j]);
-        e[j][0] = e_of<R>(ph, 0);
-        e[j][1] = e_of<R>(ph, 1);
+        const PhotonDir<R> d = photon_dir<R>(rc.k[j]);
+        e[j][0] = e_of<R>(d, 0);
+        e[j][1] = e_of<R>(d, 1);
     }
     const R n1 = rc.n1, n2 = rc.n2;
     R are[NS], aim[NS];
@@ -424,6 +458,87 @@ __device__ __forceinline__ R point_sum(const PointRec<R, N>& rc, const uint32_t*
 #pragma unroll
         for (int h = 0; h < NS; h += 2 * off) v[h] += v[h + off];
     return v[0];
+}
+
+// heget_amp2, up to kFewPoints points of a tile: the FP64 pipe takes as long for
+// one lane as for 32, and a lane with all configurations holds it for some 1500
+// instructions at n = 3.  2^n lanes of a warp share a point: tables by item as
+// at n = 4, then a lane a configuration to close them; the same operations in
+// the same order as point_sum, so the same bits, whatever the row count.
+// GB300, heget_amp2, one thread a point -> here: n = 3, 1 to 16 rows 51 -> 16 us,
+// 32 rows 52 -> 24, 64 rows 53 -> 39; n = 2, 1 row 14.6 -> 10.4, 64 rows 14.4 -> 13.4.
+// With more points than a block has such warps for, one thread a point is
+// ahead (the fused kernels' tiles are full, or share the SM with others).
+constexpr int kFewPoints = 64;
+
+template <class R, int N>
+struct FewTables {
+    static constexpr int NS = 1 << N, LP = NS;
+    static constexpr int PB = 32 / LP, NW = 8;   // points of a warp, warps
+    static constexpr int PT = (NS + 7 * N + (N == 3 ? 4 * N * (N - 1) : 0)) | 1;   // rows of a point
+    static constexpr size_t bytes = (size_t)NW * PB * PT * sizeof(Row<R>);
+    Row<R>*SD, *EA, *R1, *CL, *R2;   // as in WarpTables
+    R* EI;
+    __device__ __forceinline__ FewTables(unsigned char* smem, int point) {
+        SD = reinterpret_cast<Row<R>*>(smem) + (size_t)point * PT;
+        EA = SD + NS;
+        EI = reinterpret_cast<R*>(EA + 2 * N);
+        R1 = EA + 3 * N;
+        CL = R1 + 2 * N;
+        R2 = CL + 2 * N;
+    }
+    __device__ __forceinline__ EHel<R> e(int x) const { return EHel<R>{ld_row(EA + x), EI[x]}; }
+    static __device__ __forceinline__ EHel<R> make_e(const R* k, int lam_bit) { return e_of<R>(photon_dir<R>(k), lam_bit); }
+};
+
+template <class R, int N, int BLOCK>
+__device__ __forceinline__ void amplitude_rounds_few(unsigned char* table_smem, PointRec<R, N>* recs, int cnt,
+                                                     const uint32_t* mask) {
+    using FT = FewTables<R, N>;
+    constexpr int LP = FT::LP, PB = FT::PB, NW = FT::NW;
+    static_assert((N == 2 || N == 3) && BLOCK / 32 >= NW, "n = 2, 3");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LP;
+    if (warp < NW) {
+        const FT tb(table_smem, warp * PB + lane / LP);
+        const float wh = lane_weight<N>(mask, (unsigned)l);
+        for (int base = warp * PB; base < cnt; base += NW * PB) {
+            const int c = base + lane / LP;
+            const bool mine = c < cnt && recs[c].valid;
+            if (mine) warp_sets<R, N>(tb, recs[c], l);
+            __syncwarp();
+            if (mine) warp_ends<R, N>(tb, recs[c], l);
+            __syncwarp();
+            if constexpr (N == 3) {
+                if (mine) warp_rows<R, N>(tb, l);
+                __syncwarp();
+            }
+            R v = R(0);
+            if (mine) {
+                R ar = R(0), ai = R(0);
+                auto bit = [&](int j) { return l >> j & 1; };
+#pragma unroll
+                for (int j1 = 0; j1 < N; ++j1) {
+                    if constexpr (N == 2) {
+                        const int j2 = 1 - j1;
+                        close_row(ld_row(tb.R1 + 2 * j1 + bit(j1)), ld_row(tb.CL + 2 * j2 + bit(j2)), ar, ai);
+                    } else {
+#pragma unroll
+                        for (int t = 0; t < N - 1; ++t) {
+                            const int j2 = t + (t >= j1), j3 = 3 - j1 - j2;
+                            const int o = j1 < j2 ? bit(j1) | bit(j2) << 1 : bit(j2) | bit(j1) << 1;
+                            close_row(ld_row(tb.R2 + 4 * (j1 * (N - 1) + t) + o), ld_row(tb.CL + 2 * j3 + bit(j3)), ar, ai);
+                        }
+                    }
+                }
+                v = norm2(ar, ai) * R(sel_weight<N>(recs[c].hsel, (unsigned)l, wh));
+            }
+#pragma unroll
+            for (int off = 1; off < LP; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (c < cnt && l == 0) recs[c].ssum = v;
+            __syncwarp();
+        }
+    }
+    __syncthreads();
 }
 
 // The same contract as amplitude_rounds_lanes.
