@@ -281,11 +281,24 @@ int default_tile(int n, bool xsec) {
     // generate, three blocks fit an SM) up to n = 4, 64 at n = 5, 6 (the
     // generation spans two warps), then smaller tiles so that large-n grids
     // still cover every SM many times (a GB300 sweep of tiles and shapes).
-    // At n = 5, 48: six points a warp (a GB300 sweep at 50,001 rows: 186 us, 209
-    // with 32; FP64 at 20,001 rows 1841, 2062).
-    static const int amp2_tile[9] = {0, 0, 256, 128, 64, 48, 16, 8, 4};
+    static const int amp2_tile[9] = {0, 0, 256, 128, 64, 32, 16, 8, 4};
     static const int xsec_tile[9] = {0, 0, 128, 128, 128, 64, 64, 32, 8};
     return xsec ? xsec_tile[n] : amp2_tile[n];
+}
+
+// heget_amp2 tiles of the tree.  At n = 5, 48: six points for each warp of its
+// rounds (GB300, 50,001 rows: 186 us, 209 with 32; FP64 at 20,001 rows 1841,
+// 2062).
+int tree_amp2_tile(int n) { return n == 5 ? 48 : default_tile(n, false); }
+
+// heget_ward: rounds of block/2^n points by the whole block, so a launch takes
+// as many rounds as its busiest SM.  At n = 5 four or six a tile, whichever is
+// fewer (GB300, us, 32 | 48 points: FP32 500 rows 74 | 103, 5000 114 | 103, 60,000
+// 642 | 666; FP64 500 rows 1330 | 1985, 5000 2605 | 1987).
+int ward_tile(int n, long long npts, int num_sms) {
+    if (n != 5) return default_tile(n, false);
+    auto points = [&](int tile) { return ((npts + tile - 1) / tile + num_sms - 1) / num_sms * tile; };
+    return points(48) < points(32) ? 48 : 32;
 }
 
 // heget_amp2 tiles of the subset recursion: larger than the tree's, so that
@@ -344,7 +357,7 @@ int default_amp_launch(int n, int precision, long long npts, int num_sms, AmpLau
     if (L->shape > 0) L->block = tree_tile_shape(n, L->shape).block;
     L->tile = tile > 0 ? tile
             : xsec     ? xsec_default_tile(n, precision, alg)
-            : alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, false);
+            : alg == kAlgSubset ? subset_amp2_tile(n, precision) : tree_amp2_tile(n);
     const bool sub = alg == kAlgSubset;
     const int e = precision == HEGET_FP32
                       ? (sub ? occupancy_alg<float, kAlgSubset>(n, L->tile, &bpsm, &smem)
@@ -701,7 +714,7 @@ int heget_get_tile(const heget_ctx* ctx, int n, int precision, int kind) {
     const int t = ctx->tiles[kind][precision == HEGET_FP64][n];
     if (t > 0) return t;
     if (kind == 1) return xsec_default_tile(n, precision, ctx->alg);
-    return ctx->alg == kAlgSubset ? subset_amp2_tile(n, precision) : default_tile(n, false);
+    return ctx->alg == kAlgSubset ? subset_amp2_tile(n, precision) : tree_amp2_tile(n);
 }
 
 int heget_set_params(heget_ctx* ctx, const heget_params* p) {
@@ -802,7 +815,9 @@ int heget_ward(heget_ctx* ctx, int n, int64_t N, const double* momenta, int phot
     if (((uintptr_t)momenta & 15) != 0) return fail(HEGET_EINVAL, "momenta must be 16-byte aligned");
     DeviceGuard g(ctx->device);
     AmpLaunch L;
-    if ((r = default_amp_launch(n, precision, N, ctx->num_sms, &L, false, ctx->tiles[0][precision == HEGET_FP64][n])))
+    const int tile = ctx->tiles[0][precision == HEGET_FP64][n];
+    if ((r = default_amp_launch(n, precision, N, ctx->num_sms, &L, false,
+                                tile > 0 ? tile : ward_tile(n, N, ctx->num_sms))))
         return cuda_fail((cudaError_t)r, "occupancy");
     const Physics ph = physics_of(ctx, n);
     cudaStream_t st = (cudaStream_t)stream;
