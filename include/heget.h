@@ -378,7 +378,9 @@ int heget_amp2_escalated(heget_ctx* ctx, void* stream, int64_t* count);
  * (kind 0) or heget_xsec* (kind 1) for n photons at `precision`.  tile = 0
  * restores the default (for heget_amp2 with the subset recursion, larger
  * tiles than the tree's: 128 points at n = 4, 5 in FP32, 64 at n = 6, 32 at
- * n = 7, 8); otherwise tile must be a positive multiple of
+ * n = 7, 8; for heget_xsec* in FP64 with the subset recursion at n = 8, 8
+ * points up to 32 an SM and 16 beyond, which heget_get_tile reports);
+ * otherwise tile must be a positive multiple of
  * 256 / 2^n and at most 4096.  A tile whose shared memory exceeds the device
  * limit makes the next launch fail with HEGET_ECUDA. */
 int heget_set_tile(heget_ctx* ctx, int n, int precision, int kind, int tile);

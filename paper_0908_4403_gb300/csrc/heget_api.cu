@@ -313,14 +313,17 @@ int subset_amp2_tile(int n, int precision) {
 
 // Points per tile of the fused tile kernel.  FP64: tiles that leave room for
 // two blocks an SM (n = 4, 5), and small ones where a tile runs long (n = 8 in
-// records of rec_chunk; GB300 sweep, default -> here: tree n = 4, 262,144 points 1805 ->
-// 1598 us, n = 5, 65,536 points 2306 -> 2129; subset n = 5 1085 -> 938, n = 8, 8192
-// points 1615 with 32 -> 1413).
-int xsec_default_tile(int n, int precision, int alg) {
+// records of rec_chunk).  GB300, us, FP64: tree n = 4, tile 96 | 128: 5000 points
+// 131 | 158, 30,000 283 | 285, 262,144 1592 | 1798; n = 5, 32 | 64: 5000 points 366 |
+// 416, 65,536 2113 | 2270 (subset 162 | 194, 920 | 1072).  Subset n = 8, 8 | 16 (mean
+// of six seeds, toy PDF): 500 points 475 | 629, 2000 641 | 762, 4000 905 | 943, 6000
+// 1229 | 1240, 8192 1582 | 1530, 65,536 10,192 | 9043; at 500 GeV they cross at 5000:
+// 8 below 32 points an SM (tiles too few to hide the longest), 16 above.
+int xsec_default_tile(int n, int precision, int alg, long long npts, int num_sms) {
     if (precision == HEGET_FP64) {
         if (n == 4 && alg != kAlgSubset) return 96;
         if (n == 5) return 32;
-        if (n == 8 && alg == kAlgSubset) return 16;
+        if (n == 8 && alg == kAlgSubset) return npts < 32ll * num_sms ? 8 : 16;
     }
     return default_tile(n, true);
 }
@@ -356,7 +359,7 @@ int default_amp_launch(int n, int precision, long long npts, int num_sms, AmpLau
                                                                                         : kBlockThreads;
     if (L->shape > 0) L->block = tree_tile_shape(n, L->shape).block;
     L->tile = tile > 0 ? tile
-            : xsec     ? xsec_default_tile(n, precision, alg)
+            : xsec     ? xsec_default_tile(n, precision, alg, npts, num_sms)
             : alg == kAlgSubset ? subset_amp2_tile(n, precision) : tree_amp2_tile(n);
     const bool sub = alg == kAlgSubset;
     const int e = precision == HEGET_FP32
@@ -713,7 +716,7 @@ int heget_get_tile(const heget_ctx* ctx, int n, int precision, int kind) {
     if (!ctx || n < kMinN || n > kMaxN || (kind != 0 && kind != 1)) return -1;
     const int t = ctx->tiles[kind][precision == HEGET_FP64][n];
     if (t > 0) return t;
-    if (kind == 1) return xsec_default_tile(n, precision, ctx->alg);
+    if (kind == 1) return xsec_default_tile(n, precision, ctx->alg, LLONG_MAX, ctx->num_sms);   // (of a large call)
     return ctx->alg == kAlgSubset ? subset_amp2_tile(n, precision) : tree_amp2_tile(n);
 }
 
