@@ -179,9 +179,10 @@ hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics 
         bool fp32 = false;   // FP32 holds the event
         if (tid < cur) {
             sample_finish(S, draws[tid], ev);
-            scale = ev.rs * rambo<N>(PointRng(seed, (uint64_t)list[tid]), v);
+            ev.iM = rambo<N>(PointRng(seed, (uint64_t)list[tid]), v);
+            scale = ev.rs * ev.iM;
             wi = lw[tid];
-            fp32 = ev.rs > 1e-2 && ev.rs < 1e8;
+            fp32 = fp32_holds(ev);
             const float sf = f32_cut(fp32 ? scale : 0.0);
             // errors (u = 2^-24, components 2 u): pT 10 u; eta = ln((E + |pz|) / pT) 16 u absolute and 2 u of
             // itself; phi 16 u absolute; y = ln(ua / ub) 10 u absolute and 2 u of itself

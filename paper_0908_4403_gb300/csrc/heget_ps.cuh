@@ -514,7 +514,7 @@ __device__ __noinline__ int pass_cuts(const MomView p, double scale, u64 ua, u64
     const double s_hi = ph.sinh_eta * chy - ph.cosh_eta * shy;    // sinh(E - y)
     const double s_lo = -ph.sinh_eta * chy - ph.cosh_eta * shy;   // sinh(-E - y)
     const double pt_min = ph.pt_min / scale, pt2min = pt_min * pt_min;
-    bool ok = true;
+    bool ok = p(0, 0) == p(0, 0);   // (the comparisons on bits below do not know NaN)
     double pt2[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -590,12 +590,22 @@ __device__ __noinline__ int pass_cuts(const MomView p, double scale, u64 ua, u64
 
 // x as a float for the FP32 cut decisions: truncated towards zero (relative
 // error below 2^-23; zero below the normal float range) by three integer
-// operations on the bits.  x must be below the float range's end.
+// operations on the bits.  x must be a number below the float range's end
+// (anything else becomes some number: fp32_holds comes first).
 __device__ __forceinline__ float f32_cut(double x) {
     const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
     const unsigned int f = __funnelshift_l(lo, hi, 3) - (384u << 23);   // 9 exponent bits rebased by 896 mod 512
     const bool tiny = (hi & 0x7FFFFFFFu) < 0x38100000u;
     return tiny ? 0.0f : __uint_as_float((f & 0x7FFFFFFFu) | (hi & 0x80000000u));
+}
+
+// Whether FP32 holds an event's scale.  Not where the photons are parallel to
+// rounding: their mass M is then tiny or not a number, and so may be the
+// momenta, which f32_cut would turn into numbers.
+__device__ __forceinline__ bool fp32_holds(const EventInfo& ev) {
+    // rs in (0.01, 1e8), 1/M below 1e12, on the high words: larger for infinities, NaN and negative values
+    const unsigned r = (unsigned)__double2hiint(ev.rs), m = (unsigned)__double2hiint(ev.iM);
+    return r > 0x3F847AE1u && r < 0x4197D784u && m < 0x426D1A94u;
 }
 
 // The cut decisions in FP32 wherever FP32 settles them: the same decisions as
@@ -626,7 +636,7 @@ template <int N>
 __device__ __forceinline__ int pass_cuts_fast(const MomView& p, const EventInfo& ev, const Physics& ph) {
     constexpr float kU = 5.9604645e-8f;   // 2^-24
     const double scale = ev.rs * ev.iM;
-    if (!(ev.rs > 1e-2 && ev.rs < 1e8 && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12 &&
+    if (!(fp32_holds(ev) && ph.eta_max < 40.0 && ph.dr_min < 20.0 && ph.pt_min < 1e12 &&
           !(ph.pt_min > 0 && ph.pt_min < 1e-12) &&
           ev.ua >> 23 != 0 && ev.ub >> 23 != 0))
         return pass_cuts<N>(p, scale, ev.ua, ev.ub, ph);
