@@ -542,7 +542,7 @@ int heget_measure_fma_peak(heget_ctx* ctx, int precision, double* tflops);
  * No context is needed and nothing is allocated: no cudaMalloc, no cudaFree,
  * no allocating library routine.  The per-block partial sums that
  * heget_xsec_async keeps in the context workspace live here in a static
- * array of 4096 entries (256 KiB) that every GPU loading the library holds
+ * array of 8192 entries (512 KiB) that every GPU loading the library holds
  * until the process exits.  The caller passes the inputs and result_dev
  * (device array of sizeof(heget_xsec_result) bytes) as for
  * heget_xsec_async; params (host, may be NULL for the defaults) replaces the
@@ -550,11 +550,11 @@ int heget_measure_fma_peak(heget_ctx* ctx, int precision, double* tflops);
  *
  * It launches what heget_xsec_async launches by default (prefix tree), so
  * the results are the same bits.  Limit: a call needs one partial per block
- * of its launch; if that exceeds 4096 the call fails with HEGET_EINVAL and a
- * message giving the largest N for this n and precision.  FP32 at n <= 5
- * launches one resident wave of blocks and has no limit; otherwise N may be
- * at most 4096 x the default xsec tile (for example 262,144 points at n = 6,
- * 131,072 at n = 7 and 32,768 at n = 8 in FP32, 524,288 at n <= 4 in FP64).
+ * of its launch.  FP32 at n <= 5 launches one resident wave of blocks and has
+ * no limit; otherwise N may be at most 524,288 at n <= 4, 262,144 at n = 5, 6,
+ * 131,072 at n = 7 and 32,768 at n = 8 (4096 tiles of 128, 64, 32 and 8
+ * points), else the call fails with HEGET_EINVAL and a message giving the
+ * largest N.
  * The first call on each device looks up the array's device address
  * (cudaGetSymbolAddress) and keeps it with the CUDA context current at the
  * time; make that first call before any stream capture.  A call under

@@ -1207,7 +1207,10 @@ extern "C" int heget_xsec_batch(heget_ctx* ctx, const heget_xsec_request* reqs, 
 // reads, so nothing has to be cleared between calls.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int kNoAllocMaxBlocks = 4096;   // 4096 partials x 64 B = 256 KiB per device
+// Calls of up to 4096 tiles of default_tile points; FP64 at n = 4, 5 runs tiles
+// of three quarters and half of those, one block each, as heget_xsec_async does.
+constexpr int kNoAllocTiles = 4096;
+constexpr int kNoAllocMaxBlocks = 8192;   // 8192 partials x 64 B = 512 KiB per device
 constexpr int kNoAllocMaxDevices = 64;
 
 static __device__ __align__(256) Partial g_noalloc_partials[kNoAllocMaxBlocks];
@@ -1282,14 +1285,11 @@ extern "C" int heget_xsec_noalloc(int device, int n, uint64_t seed, int64_t i0, 
     // kernel with its default tile, whose grid bounds N
     if ((r = default_amp_launch(n, precision, N > 0 ? N : 1, sms, &L, true, 0)))
         return cuda_fail((cudaError_t)r, "occupancy");
-    // FP64 at n = 4, 5 runs smaller tiles than the range was set for: its blocks
-    // take several tiles each beyond 4096
-    const long long max_points = (long long)kNoAllocMaxBlocks * default_tile(n, true);
-    if (N > 0 && !L.ws && N > max_points)
+    const long long max_points = (long long)kNoAllocTiles * default_tile(n, true);
+    if (N > 0 && ((!L.ws && N > max_points) || L.grid > kNoAllocMaxBlocks))
         return fail(HEGET_EINVAL,
-                    "N = %lld needs more block partials than the %d of the no-allocation path (N <= %lld at n = %d)",
-                    (long long)N, kNoAllocMaxBlocks, max_points, n);
-    L.grid = std::min(L.grid, kNoAllocMaxBlocks);
+                    "N = %lld needs more block partials than the no-allocation path holds (N <= %lld at n = %d)",
+                    (long long)N, max_points, n);
     Partial* scratch = nullptr;
     if ((r = noalloc_scratch(device, &scratch))) return r;
     const Physics ph = physics_of(p, n);
