@@ -2,10 +2,10 @@
 // histograms of photon observables of the generated events.  The events of
 // nonzero weight are regenerated from the counter-based generator, 256 at a
 // time; their bins come from FP32 observables wherever FP32 settles them, and
-// the weights are added as integers (exactly) within a batch and in
-// double-double across batches and blocks, in a fixed order, so results are
-// reproducible bit for bit for a given launch shape (one resident wave, set by
-// the GPU).
+// the weights are added as integers within a batch (w exactly, w^2 rounded to
+// 55 bits or more a term) and in double-double across batches and blocks, in a
+// fixed order, so results are reproducible bit for bit for a given launch shape
+// (one resident wave, set by the GPU).
 //
 // What bounded the earlier form (GB300, five histograms of 1,048,576 events at
 // n = 4: 5480 us): 2690 FP64 instruction slots an event -- the observables'
@@ -127,8 +127,8 @@ hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics 
     constexpr int NP = N * (N - 1) / 2, NW = kHistBlock / 32;
     constexpr int E = hist_entries_max(N);
     // w: terms below 2^(53 + kTop); w^2: products of mantissas below 2^(106 + kTop2); a bin has at most
-    // E kHistBlock < 2^13 terms of a batch
-    constexpr int kTop = 60, kTop2 = 7, kSpan = 30;
+    // E kHistBlock < 2^13 terms of a batch.  The least w^2 of a pass, 2^104 2^(kTop2 - 2 kSpan), keeps 55 bits
+    constexpr int kTop = 60, kTop2 = 7, kSpan = 28;
     extern __shared__ __align__(16) unsigned char smem[];
     HistFixed* fx = reinterpret_cast<HistFixed*>(smem);
     SampleDraw* draws = reinterpret_cast<SampleDraw*>(fx + kHistBlock);
@@ -231,7 +231,7 @@ hist_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physics 
                 const unsigned __int128 m2 = (unsigned __int128)m * m;
                 const int sh = kTop2 - 2 * (em - ef);
                 fx[tid].w = fixed_of(wi, em, kTop);
-                fx[tid].w2 = (__int128)(sh >= 0 ? m2 << sh : m2 >> -sh);
+                fx[tid].w2 = (__int128)(sh >= 0 ? m2 << sh : (m2 + ((unsigned __int128)1 << (-sh - 1))) >> -sh);
             }
             for (int s = 0; s < H.nspec; ++s) {
                 const HistSpecDev& h = H.spec[s];
