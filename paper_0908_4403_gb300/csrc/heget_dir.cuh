@@ -133,6 +133,18 @@ __host__ __device__ __forceinline__ void quadrant_cos_sin(u64 f, const ulonglong
     s = a.y + ((mulhi63(a.x, sn) - (mulhi63(a.y, cm) >> 6)) >> 6);
 }
 
+// An underestimate of 1/sqrt(x), x in [xh, xh + 1) 2^-32, by less than 2^-20 of it,
+// in units of 2^-30 (FP32; rsqrtf is within 2 ulp; tested for every xh from 2^30).
+__host__ __device__ __forceinline__ u32 root_estimate(u32 xh) {
+#ifdef __CUDA_ARCH__
+    const float y = rsqrtf(__uint2float_rn(xh) * 0x1p-32f);
+    return __float2uint_rz(y * 1073741312.0f);         // y (1 - 2^-21) 2^30
+#else
+    const float y = 1.0f / __builtin_sqrtf((float)xh * 0x1p-32f);
+    return (u32)(y * 1073741312.0f);
+#endif
+}
+
 // sin theta in units of 2^-63 from a = 2^53 (1 + cos theta)/2 (odd):
 // sin^2 theta = a (2^53 - a) 2^-104, exact in 106 bits, normalised by an even
 // shift to x in [1/4, 1); with y an underestimate of 1/sqrt(x) (FP32, 2^-20)
@@ -144,13 +156,7 @@ __host__ __device__ __forceinline__ u64 sin_theta(u64 a) {
     const int ze = (clz_product(ph, pl) - 24) & ~1;
     const u64 X = top_product(ph, pl, 24 + ze);                // x 2^64
     const u32 xh = (u32)(X >> 32);
-#ifdef __CUDA_ARCH__
-    const float y = rsqrtf(__uint2float_rn(xh) * 0x1p-32f);
-    const u32 Y = __float2uint_rz(y * 1073741312.0f);         // y (1 - 2^-21) 2^30
-#else
-    const float y = 1.0f / __builtin_sqrtf((float)xh * 0x1p-32f);
-    const u32 Y = (u32)(y * 1073741312.0f);
-#endif
+    const u32 Y = root_estimate(xh);
     const u64 g = ((u64)xh * Y << 1) + ((u64)(u32)X * Y >> 31);                 // x y 2^63
     const u64 e = (X >> 2) - mulhi63(g, g);                                     // (x - g^2) 2^62, below 2^43
     const u64 d = ((u64)(u32)(e >> 32) * Y << 1) + ((u64)(u32)e * Y >> 31);     // (x - g^2) y / 2 2^62
