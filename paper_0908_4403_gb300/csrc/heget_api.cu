@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) f32_round_kernel(const double* __restrict
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ x, long long n,
                                                   Partial* __restrict__ partials) {
-    __shared__ __align__(16) Partial scratch[8];
+    __shared__ __align__(16) unsigned char scratch[reduce_scratch_bytes(256)];
     Partial a = zero_partial();
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
         const double v = x[i];
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ x, 
         a.sw2 = dd_add_d(a.sw2, v * v);
         a.ntotal += 1;
     }
-    const Partial r = block_reduce_partial<256>(a, scratch);
+    const Partial r = block_reduce_partial<256>(a, reinterpret_cast<Partial*>(scratch));
     if (threadIdx.x == 0) partials[blockIdx.x] = r;
 }
 

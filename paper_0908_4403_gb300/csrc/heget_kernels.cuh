@@ -426,6 +426,7 @@ __device__ __forceinline__ void xsec_tile(unsigned char* smem, int tile, uint64_
     __shared__ int s_cnt[BLOCK / 32];
     constexpr bool kEsc = ESC && sizeof(R) == sizeof(float);
     constexpr int TAB = table_alg<ALG, kEsc>(), kChunk = rec_chunk<R, N, TAB>();
+    static_assert(table_bytes<R, N, BLOCK, TAB, HB, G>() >= reduce_scratch_bytes(BLOCK), "the callers reduce there");
     double* stage = reinterpret_cast<double*>(smem + tile_stage_offset<R, N, BLOCK, TAB, HB, G>());
     PointRec<R, N>* recs = reinterpret_cast<PointRec<R, N>*>(smem + tile_recs_offset<R, N, BLOCK, TAB, HB, G>(tile));
     [[maybe_unused]] PassedPoint* passed = reinterpret_cast<PassedPoint*>(
@@ -598,6 +599,7 @@ xsec_escalate_kernel(uint64_t seed, long long i0, SamplerArgs S, Physics ph, int
     double* stage = reinterpret_cast<double*>(smem);
     PointRec<double, N>* recs =
         reinterpret_cast<PointRec<double, N>*>(smem + xsec_region_bytes<double, N, BLOCK, kAlgSubset>(tile));
+    static_assert(table_bytes<double, N, BLOCK, kAlgSubset>() >= reduce_scratch_bytes(BLOCK), "reduction");
     const int nb = esc.cnt[blockIdx.x];
     const size_t base = (size_t)blockIdx.x * esc.cap;
     Partial acc = zero_partial();
@@ -862,6 +864,7 @@ xsec_ws_kernel(uint64_t seed, long long i0, long long npts, SamplerArgs S, Physi
     constexpr int kWsThreads = ws_block_threads<N, ALG, ESC>();
     constexpr bool kSampler = ws_sampler(N, ALG);
     constexpr int kDrawThreads = kWsStage + 32;   // producers and the sampler's warp
+    static_assert(ws_recs_offset<R, N, ALG, table_alg<ALG, ESC>()>() >= reduce_scratch_bytes(kWsThreads), "reduction");
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int TAB = table_alg<ALG, ESC>();
     PointRec<R, N>* ring = reinterpret_cast<PointRec<R, N>*>(smem + ws_recs_offset<R, N, ALG, TAB>());

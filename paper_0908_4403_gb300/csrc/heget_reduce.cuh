@@ -127,33 +127,39 @@ __device__ __forceinline__ Partial zero_partial() {
 
 // Sum of the per-thread partials of a block: the largest exponents of all
 // threads, the warps' sums as integers aligned to them, one thread adds those.
-// Uses `scratch` (BLOCK/32 Partials of shared memory, 16-byte aligned); result
-// valid in thread 0.  All threads must call it.
+// Uses `scratch` (reduce_scratch_bytes(BLOCK) of shared memory, 16-byte
+// aligned: the sums and, behind them, the exponents of the warps); result
+// valid in thread 0.  All threads must call it.  (No shared memory of its own:
+// the largest tiles leave 32 bytes of a block's.)
 struct alignas(16) WarpSums {
     __int128 v[2];
     long long c[4];
 };
 static_assert(sizeof(WarpSums) == sizeof(Partial), "the scratch holds one per warp");
 
+__host__ __device__ constexpr size_t reduce_scratch_bytes(int block) {
+    return block / 32 * (sizeof(Partial) + 2 * sizeof(int));
+}
+
 template <int BLOCK>
 __device__ __forceinline__ Partial block_reduce_partial(Partial a, Partial* scratch) {
     static_assert(BLOCK % 32 == 0 && BLOCK <= 1024, "whole warps");
     constexpr int NW = BLOCK / 32;
     constexpr int kTop = 61;   // 2 BLOCK <= 2048 terms of a sum below 2^(53 + kTop)
-    __shared__ int s_em[2][NW];
     WarpSums* sums = reinterpret_cast<WarpSums*>(scratch);
+    int* s_em = reinterpret_cast<int*>(scratch + NW);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int em[2] = {(int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a.sw)),
                  (int)__reduce_max_sync(0xffffffffu, (unsigned)exponent_field(a.sw2))};
     if (lane == 0) {
-        s_em[0][warp] = em[0];
-        s_em[1][warp] = em[1];
+        s_em[warp] = em[0];
+        s_em[NW + warp] = em[1];
     }
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-        em[0] = max(em[0], s_em[0][w]);
-        em[1] = max(em[1], s_em[1][w]);
+        em[0] = max(em[0], s_em[w]);
+        em[1] = max(em[1], s_em[NW + w]);
     }
     WarpSums t{{fixed_of(a.sw, em[0], kTop), fixed_of(a.sw2, em[1], kTop)}, {a.npass, a.ntotal, a.ntries, a.nesc}};
 #pragma unroll
