@@ -172,9 +172,13 @@ struct MeetTables {
         return LV(g, p) + J0 + J1 + (((MK - 1 - k) & 1) ? K0 : 0);
     }
     __device__ __forceinline__ Row<R>* RV(int g, int p) const { return LV(g, p) + J0 + J1 + K0 + K1; }
-    __device__ __forceinline__ R* XA(int g, int p) const {
-        return XA_OVER ? reinterpret_cast<R*>(LV(g, p) + J0)
-                       : reinterpret_cast<R*>(base + (size_t)g * GB + (size_t)PG * PT * sizeof(Row<R>)) + p * XAP;
+    // amplitudes of contraction group u of a point: overlaid, the point's own; else point-minor, so that the lanes
+    // of a warp, taking consecutive points, spread over the banks (GB300, heget_amp2 in FP32, a place per point ->
+    // here: 1,048,576 rows at n = 2 412 -> 333 us, n = 3 865 -> 735)
+    __device__ __forceinline__ R* XA(int g, int p, int u) const {
+        return XA_OVER ? reinterpret_cast<R*>(LV(g, p) + J0) + (((size_t)u << CB) * CT * 2)
+                       : reinterpret_cast<R*>(base + (size_t)g * GB + (size_t)PG * PT * sizeof(Row<R>)) +
+                             ((((size_t)u * PG + p) << CB) * CT * 2);
     }
 };
 
@@ -543,8 +547,9 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
             const int rc = min(PG, cnt - base);
             const PointRec<R, N>* rb = recs + base;
             // photon and set data (n = 2 has no larger sets: its currents come
-            // straight from the records, a phase and a barrier less -- GB300, FP32
-            // heget_amp2 of 12,001 rows 31 us, 35 with the tables; 262,144 rows 128, 140)
+            // straight from the records, a phase and a barrier less -- GB300,
+            // heget_amp2, with the tables -> here: FP32 5000 rows 31 -> 27 us,
+            // 262,144 rows 119 -> 107, FP64 2051 -> 1816)
             constexpr bool kDirect = N == 2;
             if constexpr (!kDirect) {
                 meet_photons_and_sets(tb, g, lid, rb, rc);
@@ -602,11 +607,11 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
                 }
                 if (c0 + CH < CM) meet_sync<BAR, BLOCK, GBAR0, GTH, G>(g);   // before the next chunk's currents
             }
-            // the groups' amplitudes, configuration-major (entry (u 2^CB + b) CT + hi
-            // of the point for lambda = (hi << CB) | b): a warp's lanes store
+            // the groups' amplitudes, configuration-major (entry b CT + hi of the
+            // group and point for lambda = (hi << CB) | b): a warp's lanes store
             // consecutive words
             if (mine) {
-                R* xa = tb.XA(g, p) + ((size_t)gt << CB) * CT * 2 + (size_t)hi * 2;
+                R* xa = tb.XA(g, p, gt) + (size_t)hi * 2;
 #pragma unroll
                 for (int b = 0; b < (1 << CB); ++b) {
                     using V2 = typename std::conditional<sizeof(R) == sizeof(float), float2, double2>::type;
@@ -631,7 +636,7 @@ __device__ __noinline__ void amplitude_rounds_meet(unsigned char* table_smem, Po
                         R ar = R(0), ai = R(0);
 #pragma unroll
                         for (int u = 0; u < GT; ++u) {
-                            const R* a = tb.XA(g, q) + (((size_t)u << CB) + b) * CT * 2 + (size_t)hh * 2;
+                            const R* a = tb.XA(g, q, u) + ((size_t)b * CT + hh) * 2;
                             ar += a[0];
                             ai += a[1];
                         }
