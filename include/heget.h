@@ -247,9 +247,10 @@ typedef struct {
  * Every request is cut into point tiles: the context's xsec tile if set
  * (heget_set_tile), else with the tree the tiles heget_xsec uses on the
  * plain (non-warp-specialised) path, with the subset recursion tiles of 128
- * points (FP32: 64 from n = 5; FP64: 64 at n = 4, 16 at
- * n = 5, 8 from n = 6), the largest that let two blocks share an SM.  The
- * kernel is compiled once per algorithm.  The tiles of all requests, whatever
+ * points (FP32: 64 from n = 5; FP64: 32 at n = 5, 64 at n = 6, 32 at n = 7
+ * and 16 at n = 8).  Two blocks share an SM, except in FP64 from n = 6 with the
+ * subset recursion: one block, and one such request sets the shared memory of
+ * the whole FP64 launch.  The kernel is compiled once per algorithm.  The tiles of all requests, whatever
  * their n and N, form one work list that a single kernel walks, and each
  * request's tile partials are combined in tile order, so a request's result
  * does not depend on what else is in the batch.  reqs: host array of `count`
@@ -295,10 +296,11 @@ typedef struct {
  * histograms with at most HEGET_HIST_MAX_BINS bins in all.  out: device
  * doubles, for each spec in order its nbins + 2 bins (underflow, the bins,
  * overflow), each as (sum w, sum w^2): 2 sum (nbins + 2) values, written
- * (zeros for N = 0).  Each block sums its tiles' entries per bin in a fixed
- * order and folds the tile sums into double-double sums, combined in block
- * order: results are reproducible bit for bit on a given GPU model (the
- * grid is one resident wave).  EINVAL for bad specs, n, N, sampler or NULL
+ * (zeros for N = 0).  Each block packs its events of nonzero weight into
+ * batches, adds a batch's entries per bin as integers (w exactly, w^2 with 55
+ * bits or more of each term) and folds them into double-double sums, which are
+ * combined across blocks as integers: results are reproducible bit for bit on a
+ * given GPU model (the grid is one resident wave).  EINVAL for bad specs, n, N, sampler or NULL
  * arrays (N > 0). */
 int heget_hist(heget_ctx* ctx, int n, uint64_t seed, int64_t i0, int64_t N,
                const heget_sampler* sampler, const double* w,

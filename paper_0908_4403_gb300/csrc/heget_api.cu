@@ -287,8 +287,9 @@ int default_tile(int n, bool xsec) {
 }
 
 // heget_amp2 tiles of the tree.  At n = 5, 48: six points for each warp of its
-// rounds (GB300, 50,001 rows: 186 us, 209 with 32; FP64 at 20,001 rows 1841,
-// 2062).
+// rounds (GB300, us, 32 | 48 | 64 points: FP32 5000 rows 43 | 41 | 49, 50,001 209 |
+// 188 | 198, 200,000 756 | 688 | 656; FP64 5000 rows 623 | 471 | 623, 50,001 3376 |
+// 3273 | 3709; 500 rows, less than a tile an SM, 32 | 39 | 47 and 318 | 471 | 623).
 int tree_amp2_tile(int n) { return n == 5 ? 48 : default_tile(n, false); }
 
 // heget_ward: rounds of block/2^n points by the whole block, so a launch takes
@@ -511,9 +512,12 @@ size_t batch_tile_smem(int n, int precision, int alg, int tile) {
 
 int batch_default_tile(int n, int precision, int alg) {
     // subset recursion: the largest tile whose block (records, staging and
-    // the recursion's tables) still lets two blocks share an SM, up to 128
+    // the recursion's tables) still lets two blocks share an SM, up to 128;
+    // FP64 from n = 6: one block (181, 135, 154 KB), rec_chunk records of a tile
+    // at a time.  (GB300, 24 mixed requests of up to 2000 | 8000 | 30,000 | 65,536
+    // points, with FP64 tiles 64, 16, 8, 8, 8 from n = 4 -> here: 1255 -> 1194, 1576 ->
+    // 1285, 2785 -> 1856, 4860 -> 3248 us, the round tables' gains included.)
     static const int sub32[9] = {0, 0, 128, 128, 128, 64, 64, 64, 64};
-    // (FP64 from n = 6: rec_chunk records of a larger tile at a time)
     static const int sub64[9] = {0, 0, 128, 128, 128, 32, 64, 32, 16};
     if (alg != kAlgSubset) return default_tile(n, true);
     return precision == HEGET_FP64 ? sub64[n] : sub32[n];

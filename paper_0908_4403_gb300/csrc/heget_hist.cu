@@ -11,7 +11,7 @@
 // n = 4: 5480 us): 2690 FP64 instruction slots an event -- the observables'
 // asinh, atan2, log and square roots in FP64, bin sums with one active lane an
 // FP64 instruction, and the events of zero weight, generated and dropped.
-// Here, 97 slots (41 % of the FP64 pipe) and 154 warp instructions an event: 532
+// Here, 97 slots (41 % of the FP64 pipe) and 154 warp instructions an event: 511
 // us, bound by the barriers between the passes of a batch (six a histogram).
 #include <algorithm>
 #include <cmath>

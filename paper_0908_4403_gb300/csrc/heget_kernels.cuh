@@ -807,11 +807,12 @@ __host__ __device__ constexpr int ws_stage(int n, int alg) {
 }
 
 // Whether a warp of its own draws for the producers (warp_draws over a whole
-// stage).  GB300, one million points (64 K at n = 8), consumers drawing ->
-// sampler's warp: n = 3 519 -> 443 us, n = 4 630 -> 612, subset n = 4 1006 -> 942, n
-// = 8 685 -> 665.  At n = 2 one warp cannot keep up with the producers (309 ->
-// 349), and at n = 5, 6 32 more threads would cost the consumers registers (two
-// blocks of 352 threads leave 93).
+// stage).  GB300, us, consumers drawing -> sampler's warp, 1,048,576 points (65,536
+// from n = 7), toy PDF: n = 3 516 -> 450, n = 4 629 -> 611, subset n = 4 873 -> 804,
+// n = 7 382 -> 370, n = 8 660 -> 616; 10,007 points within 1 us, n = 8 201 -> 195.
+// At n = 2 one warp cannot keep up with the producers (306 -> 365), and at n = 5,
+// 6 32 more threads would cost the consumers registers (two blocks of 352 threads
+// leave 93).
 __host__ __device__ constexpr bool ws_sampler(int n, int alg) { return n == 3 || n == 4 || (n >= 7 && alg == 1); }
 
 __device__ __forceinline__ void named_sync(int id, int count) {

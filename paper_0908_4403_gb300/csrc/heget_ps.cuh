@@ -429,8 +429,9 @@ __device__ __forceinline__ double recip_series(double x) {
 // frame of their sum.
 //
 // GB300, FP64 instructions a point, before -> after: 403 -> 154 at n = 4, 500,000
-// phase-space points at n = 5 454 -> 226 us (unrolling the loops by 2 or 4: no
-// gain, more instruction-cache misses).  True error of the momenta (against
+// phase-space points at n = 5 454 -> 226 us (230 now, with the guards for parallel
+// photons; unrolling the loops by 2 or 4: no gain, more instruction-cache
+// misses).  True error of the momenta (against
 // quad precision, 2-norm): n = 5 2.71e-16 -> 2.69e-16, n = 2 3.2e-14 -> 2.4e-14.
 template <int N>
 __device__ __forceinline__ double rambo(const PointRng& rng, const MomView& v) {
@@ -626,7 +627,7 @@ __device__ __forceinline__ bool fp32_holds(const EventInfo& ev) {
 // (90 of 545 at n = 4) at 64 cycles each per warp; these cost about 70 n + 20
 // n (n - 1) / 2 FP32 and integer instructions at 1 - 2 cycles.  GB300, before ->
 // after: n = 4 step of 1,048,576 points 1123 -> 1012 us, phase space of 500,000
-// points at n = 5 668 -> 454 us.
+// points at n = 5 668 -> 454 us (this form alone; both are faster by now: rambo).
 //
 // The momenta are in RAMBO's units (total M, of the order of n), which FP32
 // holds; pT is compared in GeV.  Energies, pT cuts, boosts (u below 2^-30), e^2E

@@ -18,9 +18,10 @@
 // 1,048,576 points 661 -> 384 and 1027 -> 644 us (its consumers were what the FP64
 // producers waited for); heget_amp2 of 50,001 rows at n = 5 5013 -> 2500 and 322 ->
 // 190 us; FP64 at n = 4, 262,144 points 3030 -> 2346 us, and 1806 with the orders
-// of a pair added first (warp_add_orders).  What bounds it now: fixed
-// latencies and the instruction cache (issue 51 %, FMA pipe 31 %, FP64 pipe 47 %
-// of the fused n = 4 kernel).
+// of a pair added first (warp_add_orders).  (These rounds alone; with the
+// sampler's warp and the FP64 tiles the calls take 611, 187 and 1587 us.)  What
+// bounds it now: fixed latencies and the instruction cache (issue 51 %, FMA pipe
+// 31 %, FP64 pipe 47 % of the fused n = 4 kernel).
 #pragma once
 
 #include "heget_amp.cuh"
